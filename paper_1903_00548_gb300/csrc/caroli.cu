@@ -140,11 +140,11 @@ extern "C" int pwqt_transmission_caroli(pwqt_ctx* c, int sys, int n_E, const dou
         PWQT_CUDA(c, cudaMemcpyAsync(jobs_d.p, jobs.data(), sizeof(SweepJob) * nb, cudaMemcpyHostToDevice, st));
         PWQT_CUDA(c, cudaMemcpyAsync(sig_d.p, sig.data(), sizeof(double2*) * 2 * nb, cudaMemcpyHostToDevice, st));
         SweepSys sy{n, N, c->M0.as<double2>(), c->M1.as<double2>(), s.HV0.as<double2>(), s.HV1.as<double2>()};
-        launch_sweep_fp64(sy, jobs_d.as<SweepJob>(), nb, st);
+        c->launches += launch_sweep_fp64(sy, jobs_d.as<SweepJob>(), jobs.data(), nb, st);
         const int gblocks = (int)std::min<size_t>((nn + 255) / 256, 1024);
         k_broadening<<<dim3(gblocks, nb), 256, 0, st>>>(n, sig_d.as<const double2*>(), Gs);
         k_broadening<<<dim3(gblocks, nb), 256, 0, st>>>(n, sig_d.as<const double2*>() + nb, Gd);
-        c->launches += 3;
+        c->launches += 2;
         PWQT_CUDA(c, cudaGetLastError());
         // G_{N1}: the solution columns of the last node, row-major with leading dimension 2n.
         // cuBLAS is column-major: a row-major matrix read in place is its transpose, so

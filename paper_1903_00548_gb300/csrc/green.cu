@@ -80,8 +80,7 @@ extern "C" int pwqt_green_diagonal(pwqt_ctx* c, int sys, int n_E, const double* 
         PWQT_TRY(ensure(c, jobs_d, sizeof(SweepJob) * nb));
         PWQT_CUDA(c, cudaMemcpyAsync(jobs_d.p, jobs.data(), sizeof(SweepJob) * nb, cudaMemcpyHostToDevice, st));
         SweepSys sy{n, N, c->M0.as<double2>(), c->M1.as<double2>(), s.HV0.as<double2>(), s.HV1.as<double2>()};
-        launch_green_fp64(sy, jobs_d.as<SweepJob>(), nb, st);
-        c->launches++;
+        c->launches += launch_green_fp64(sy, jobs_d.as<SweepJob>(), jobs.data(), nb, st);
         PWQT_CUDA(c, cudaGetLastError());
         std::vector<int> sk(nb);
         PWQT_CUDA(c, cudaMemcpyAsync(node_dos + (size_t)e0 * N, dos, sizeof(double) * N * nb, cudaMemcpyDeviceToHost, st));

@@ -15,43 +15,57 @@ namespace pwqt {
 // T_gamma = sum_{mu traveling out at d} |(P_d c_N)_{mu gamma}|^2 v_mu / v_gamma  (Eq. transmission)
 // R_gamma with the injected part removed at node 1, T_ds for drain-injected modes,
 // node density n[i][c] = sum_{gamma in c} (2/|v_gamma|) sum_alpha |c_{i alpha gamma}|^2.
-__global__ void k_observables(int n, int N, const ObsJob* __restrict__ jobs) {
-    const ObsJob J = jobs[blockIdx.x];
+// ntd ms + nts m inner products of length n per energy, FP64-bound: dealt out to OBS_CTAS
+// CTAs per energy, a warp per out-mode with its lanes along the injected modes (one
+// energy's CTA took 0.6 ms at n = 128 and 77 modes when it did them alone).  The CTAs'
+// sums meet in the outputs, which the caller has zeroed.
+constexpr int OBS_CTAS = 16;
+__global__ void __launch_bounds__(256) k_observables(int n, int N, const ObsJob* __restrict__ jobs) {
+    const ObsJob& J = jobs[blockIdx.x];
     const int m = J.ms + J.md;
-    __shared__ double acc[3];
-    if (threadIdx.x < 3) acc[threadIdx.x] = 0.0;
-    __syncthreads();
     const double2* cN = J.C + (size_t)(N - 1) * J.node_stride;
     const double2* c1 = J.C;
     double t_loc = 0, r_loc = 0, tds_loc = 0;
-    // transmission s -> d
-    for (int t = threadIdx.x; t < J.ntd * J.ms; t += blockDim.x) {
-        int mu = t / J.ms, g = t % J.ms;
-        double2 a = make_double2(0, 0);
-        for (int k = 0; k < n; ++k) cfma(a, J.P_d[(size_t)mu * n + k], cN[(size_t)k * J.row_stride + g]);
-        t_loc += cnorm2(a) * J.v_out_d[mu] / J.v_in_s[g];
-    }
-    // reflection at s and transmission d -> s
-    for (int t = threadIdx.x; t < J.nts * m; t += blockDim.x) {
-        int mu = t / m, g = t % m;
-        double2 a = make_double2(0, 0);
+    const int lane = threadIdx.x & 31, gs = (J.ms + 31) / 32, gm = (m + 31) / 32;
+    const int items_t = J.ntd * gs, items = items_t + J.nts * gm;
+    for (int q = blockIdx.y * 8 + (threadIdx.x >> 5); q < items; q += OBS_CTAS * 8) {
+        const bool td = q < items_t;                         // transmission s -> d, else back at the source
+        const int p = td ? q : q - items_t, mu = td ? p / gs : p / gm, g = (td ? p % gs : p % gm) * 32 + lane;
+        if (g >= (td ? J.ms : m)) continue;
+        const double2* P = (td ? J.P_d : J.P_s) + (size_t)mu * n;
+        const double2* c = (td ? cN : c1) + g;
+        const bool inj = !td && g < J.ms;                    // remove the injected part
+        double rr = 0, ii = 0, ri = 0, ir = 0;
+#pragma unroll 4
         for (int k = 0; k < n; ++k) {
-            double2 v = c1[(size_t)k * J.row_stride + g];
-            if (g < J.ms) v = csub(v, J.cin_s[(size_t)k * J.ms + g]);
-            cfma(a, J.P_s[(size_t)mu * n + k], v);
+            const double2 a = P[k];
+            double2 b = c[(size_t)k * J.row_stride];
+            if (inj) b = csub(b, J.cin_s[(size_t)k * J.ms + g]);
+            rr = fma(a.x, b.x, rr);
+            ii = fma(a.y, b.y, ii);
+            ri = fma(a.x, b.y, ri);
+            ir = fma(a.y, b.x, ir);
         }
-        if (g < J.ms) r_loc += cnorm2(a) * J.v_out_s[mu] / J.v_in_s[g];
-        else tds_loc += cnorm2(a) * J.v_out_s[mu] / J.v_in_d[g - J.ms];
+        const double f = cnorm2(make_double2(rr - ii, ri + ir));
+        if (td) t_loc += f * J.v_out_d[mu] / J.v_in_s[g];
+        else if (g < J.ms) r_loc += f * J.v_out_s[mu] / J.v_in_s[g];
+        else tds_loc += f * J.v_out_s[mu] / J.v_in_d[g - J.ms];
     }
-    atomicAdd(&acc[0], t_loc);
-    atomicAdd(&acc[1], r_loc);
-    atomicAdd(&acc[2], tds_loc);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        *J.T = acc[0];
-        *J.R = acc[1];
-        *J.T_ds = acc[2];
+    for (int o = 16; o > 0; o >>= 1) {
+        t_loc += __shfl_down_sync(0xffffffffu, t_loc, o);
+        r_loc += __shfl_down_sync(0xffffffffu, r_loc, o);
+        tds_loc += __shfl_down_sync(0xffffffffu, tds_loc, o);
     }
+    if (lane == 0) {
+        if (t_loc != 0.0) atomicAdd(J.T, t_loc);
+        if (r_loc != 0.0) atomicAdd(J.R, r_loc);
+        if (tds_loc != 0.0) atomicAdd(J.T_ds, tds_loc);
+    }
+}
+
+__global__ void k_observables_zero(const ObsJob* __restrict__ jobs, int nb) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < nb) *jobs[b].T = *jobs[b].R = *jobs[b].T_ds = 0.0;
 }
 
 // node density of node blockIdx.x, energy blockIdx.y: one CTA sums the n x m
@@ -90,51 +104,12 @@ __global__ void __launch_bounds__(256) k_node_density(int n, const ObsJob* __res
 }
 
 void launch_observables(int n, int N, const ObsJob* jobs, int nb, cudaStream_t st) {
-    k_observables<<<nb, 256, 0, st>>>(n, N, jobs);
+    k_observables_zero<<<(nb + 127) / 128, 128, 0, st>>>(jobs, nb);
+    k_observables<<<dim3(nb, OBS_CTAS), 256, 0, st>>>(n, N, jobs);
     k_node_density<<<dim3(N, nb), 256, 0, st>>>(n, jobs);
 }
 
-// ---------------------------------------------------------------- FP64 residual
-// r_i = b_i - (L_i c_{i-1} + D_i c_i + U_i c_{i+1}) (FP64), per column sums of |r|^2 and |b|^2.
-__global__ void k_residual_fp64(SweepSys sys, const ResJob* __restrict__ jobs) {
-    const ResJob J = jobs[blockIdx.y];
-    const int n = sys.n, N = sys.N, m = J.ms + J.md;
-    const int i = blockIdx.x;
-    if (m == 0) return;
-    const double E = J.E;
-    const double2* ci = J.C + (size_t)i * J.node_stride;
-    const double2* cm1 = i > 0 ? J.C + (size_t)(i - 1) * J.node_stride : nullptr;
-    const double2* cp1 = i < N - 1 ? J.C + (size_t)(i + 1) * J.node_stride : nullptr;
-    const double2* HV0b = J.HV0 ? J.HV0 : sys.HV0;
-    const double2* HV1b = J.HV1 ? J.HV1 : sys.HV1;
-    const double2* HV0 = HV0b + (size_t)i * n * n;
-    const double2* HV1 = HV1b + (size_t)i * n * n;
-    const double2* HVm = i > 0 ? HV1b + (size_t)(i - 1) * n * n : nullptr;
-    for (int t = threadIdx.x; t < n * m; t += blockDim.x) {
-        int r = t / m, g = t % m;
-        double2 acc = make_double2(0, 0);
-        for (int k = 0; k < n; ++k) {
-            size_t rk = (size_t)r * n + k;
-            double2 d = csub(cscale(sys.M0[rk], E), HV0[rk]);
-            if (i == 0) d = csub(d, J.sig_s[rk]);
-            if (i == N - 1) d = csub(d, J.sig_d[rk]);
-            cfma(acc, d, ci[(size_t)k * J.row_stride + g]);
-            if (cp1) cfma(acc, csub(cscale(sys.M1[rk], E), HV1[rk]), cp1[(size_t)k * J.row_stride + g]);
-            if (cm1) {
-                size_t kr = (size_t)k * n + r;
-                cfma(acc, cconj(csub(cscale(sys.M1[kr], E), HVm[kr])), cm1[(size_t)k * J.row_stride + g]);
-            }
-        }
-        double2 b = make_double2(0, 0);
-        if (i == 0 && g < J.ms) b = J.rhs_s[(size_t)r * J.ms + g];
-        if (i == N - 1 && g >= J.ms) b = J.rhs_d[(size_t)r * J.md + (g - J.ms)];
-        double2 res = csub(b, acc);
-        if (J.Rout) J.Rout[(size_t)i * J.r_node_stride + (size_t)r * J.r_row_stride + g] = res;
-        atomicAdd(&J.rn2[g], cnorm2(res));
-        atomicAdd(&J.bn2[g], cnorm2(b));
-    }
-}
-
+// ---------------------------------------------------------------- residual
 __global__ void k_residual_finish(const ResJob* __restrict__ jobs, int nb, const int* __restrict__ active) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nb || (active && !active[b])) return;
@@ -152,12 +127,6 @@ __global__ void k_residual_finish(const ResJob* __restrict__ jobs, int nb, const
 
 void launch_residual_finish(const ResJob* jobs, int nb, cudaStream_t st, const int* active) {
     k_residual_finish<<<(nb + 127) / 128, 128, 0, st>>>(jobs, nb, active);
-}
-
-void launch_residual_fp64(const SweepSys& sys, const ResJob* jobs, int nb, cudaStream_t st) {
-    dim3 grid(sys.N, nb);
-    k_residual_fp64<<<grid, 256, 0, st>>>(sys, jobs);
-    launch_residual_finish(jobs, nb, st);
 }
 
 __global__ void k_fill_int(int* p, int v, int cnt) {
@@ -296,8 +265,7 @@ int solve_batch(pwqt_ctx* c, System& s, int nE, const double* E, int precision, 
                                  o.iters + g0, gs, precision == PWQT_MIXED, *L, sys_of ? sys_of + g0 : nullptr));
         } else {
             if (c->profile) PWQT_CUDA(c, cudaEventRecord(c->ev0, gs));
-            launch_sweep_fp64(sys, jobs_d.as<SweepJob>(), gn, gs);
-            c->launches++;
+            c->launches += launch_sweep_fp64(sys, jobs_d.as<SweepJob>(), jobs.data(), gn, gs);
             if (c->profile) {
                 PWQT_CUDA(c, cudaEventRecord(c->ev1, gs));
                 PWQT_CUDA(c, cudaEventSynchronize(c->ev1));
@@ -308,7 +276,7 @@ int solve_batch(pwqt_ctx* c, System& s, int nE, const double* E, int precision, 
                 c->prof_flops += (56.0 / 3.0) * (double)N * n * n * (double)n * gn;
             }
             PWQT_CUDA(c, cudaGetLastError());
-            launch_residual_fp64(sys, res_d.as<ResJob>(), gn, gs);
+            launch_residual_fp64(sys, res_d.as<ResJob>(), (int)maxm, gn, gs);
             c->launches += 2;
             if (o.iters) {
                 k_fill_int<<<(gn + 127) / 128, 128, 0, gs>>>(o.iters + g0, 0, gn);
@@ -316,7 +284,7 @@ int solve_batch(pwqt_ctx* c, System& s, int nE, const double* E, int precision, 
             }
         }
         launch_observables(n, N, obs_d.as<ObsJob>(), gn, gs);
-        c->launches += 2;
+        c->launches += 3;
         PWQT_CUDA(c, cudaGetLastError());
         PWQT_CUDA(c, cudaStreamSynchronize(gs));
         return PWQT_OK;

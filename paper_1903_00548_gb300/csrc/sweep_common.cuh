@@ -45,11 +45,13 @@ struct ObsJob {
     double* T; double* R; double* T_ds; double* node_n;   // node_n: N x 2
 };
 
-void launch_sweep_fp64(const SweepSys& sys, const SweepJob* jobs, int nb, cudaStream_t st);
+// `host` is the host's copy of the job table (column counts size the launches); both
+// return the number of kernels launched.
+int launch_sweep_fp64(const SweepSys& sys, const SweepJob* jobs, const SweepJob* host, int nb, cudaStream_t st);
 // Diagonal blocks of G = [E M - H - Sigma]^{-1} by the recursive Green's-function
 // recursion over the nodes (jobs with ms = n, md = 0; XY holds N x n x 2n):
 // on return XY_i = [* | G_ii] and dos[i] = -(2/pi) Im Tr G_ii.
-void launch_green_fp64(const SweepSys& sys, const SweepJob* jobs, int nb, cudaStream_t st);
+int launch_green_fp64(const SweepSys& sys, const SweepJob* jobs, const SweepJob* host, int nb, cudaStream_t st);
 void launch_observables(int n, int N, const ObsJob* jobs, int nb, cudaStream_t st);
 // rank-m updates of the density matrix from one batch of solved energies (density.cu);
 // E and the weights in d.w are this batch's

@@ -28,7 +28,8 @@ struct ResJob {
     double* resid;             // max over columns of ||r|| / ||b||
 };
 
-void launch_residual_fp64(const SweepSys& sys, const ResJob* jobs, int nb, cudaStream_t st);
+// m: the largest column count of the batch
+void launch_residual_fp64(const SweepSys& sys, const ResJob* jobs, int m, int nb, cudaStream_t st);
 // the same residual in float-float arithmetic on the FP32 pipes (~48-bit significand):
 // blocks pre-split into (hi, lo) float pairs, stored as float4 (re_hi, re_lo, im_hi, im_lo)
 struct ResidualFF {
