@@ -277,16 +277,20 @@ __global__ void __launch_bounds__(NT) k_sweep_fp64(SweepSys sys, const SweepJob*
 
 // ---------------------------------------------------------------- tile product
 // acc = sum_k A(r0 + ., k) B(k, c0 + .) over a T x T tile, T = 16 R: 256 threads, R x R
-// outputs each, four real accumulators per output (independent chains: an FP64 FMA takes
-// 64 cycles).  A and B are read through functors that return zero outside the operands;
-// the next 16 k are fetched while the current ones are multiplied.
+// outputs each.  A and B are read through functors that return zero outside the operands;
+// the next 16 k are fetched while the current ones are multiplied.  A warp holds 2 R rows and
+// skips those past M and the column halves past Nc: an FP64 instruction costs a warp 64
+// cycles however few of its lanes count.
 template <int R> struct TileMem { double2 a[16 * R][17], b[16][16 * R + 1]; };
 
 template <int R, class AF, class BF>
-__device__ __forceinline__ void tile_product(TileMem<R>& sm, int r0, int c0, int K, AF A, BF B, double2 (&out)[R][R]) {
+__device__ __forceinline__ void tile_product(TileMem<R>& sm, int r0, int c0, int M, int Nc, int K, AF A, BF B, double2 (&out)[R][R]) {
     constexpr int T = 16 * R;
     const int t = threadIdx.x, tx = t % 16, ty = t / 16;
-    double rr[R][R] = {}, ii[R][R] = {}, ri[R][R] = {}, ir[R][R] = {};
+#pragma unroll
+    for (int x = 0; x < R; ++x)
+#pragma unroll
+        for (int y = 0; y < R; ++y) out[x][y] = make_double2(0, 0);
     double2 fa[R], fb[R];
     auto fetch = [&](int k0) {
 #pragma unroll
@@ -307,25 +311,20 @@ __device__ __forceinline__ void tile_product(TileMem<R>& sm, int r0, int c0, int
         }
         __syncthreads();
         if (k0 + 16 < K) fetch(k0 + 16);
+        const int ke = min(16, K - k0);
 #pragma unroll 4
-        for (int k = 0; k < 16; ++k)
+        for (int k = 0; k < ke; ++k)
 #pragma unroll
             for (int x = 0; x < R; ++x) {
+                if (r0 + 16 * x + (ty & ~1) >= M) continue;
                 const double2 a = sm.a[ty + 16 * x][k];
 #pragma unroll
                 for (int y = 0; y < R; ++y) {
-                    const double2 b = sm.b[k][tx + 16 * y];
-                    rr[x][y] = fma(a.x, b.x, rr[x][y]);
-                    ii[x][y] = fma(a.y, b.y, ii[x][y]);
-                    ri[x][y] = fma(a.x, b.y, ri[x][y]);
-                    ir[x][y] = fma(a.y, b.x, ir[x][y]);
+                    if (c0 + 16 * y >= Nc) continue;
+                    cfma(out[x][y], a, sm.b[k][tx + 16 * y]);
                 }
             }
     }
-#pragma unroll
-    for (int x = 0; x < R; ++x)
-#pragma unroll
-        for (int y = 0; y < R; ++y) out[x][y] = make_double2(rr[x][y] - ii[x][y], ri[x][y] + ir[x][y]);
 }
 
 __device__ __forceinline__ const double2* hv0_of(const SweepSys& s, const SweepJob& J, int i) {
@@ -370,7 +369,7 @@ __global__ void __launch_bounds__(256) k_node(SweepSys sys, const SweepJob* __re
             return cconj(csub(cscale(M1[q], E), HVm[q]));
         };
         auto B = [&](int k, int c) { return c < pc ? P[(size_t)k * w + c] : make_double2(0, 0); };
-        tile_product<R>(sm, r0, c0, n, A, B, acc);
+        tile_product<R>(sm, r0, c0, n, cols, n, A, B, acc);
     }
     const double2* HV0 = hv0_of(sys, J, i);
 #pragma unroll
@@ -405,10 +404,15 @@ struct Where64 {
 
 // ---------------------------------------------------------------- solve for [X_i | y_i]
 // Columns [c0, c0 + CB) of P [U_i | y] through L and U (unit lower; the factors in S): the
-// columns stay in shared memory, the factors pass through it in panels of 16 columns.  The
-// 16 x 16 diagonal systems run in half-warps (lane = row, one column each).
-__host__ __device__ constexpr int solve_panel_ld() { return 17; }
-size_t solve_smem(int n, int cb) { return sizeof(double2) * ((size_t)n * cb + (size_t)n * solve_panel_ld()); }
+// columns stay in shared memory, the factors pass through it in panels of 8 columns, the
+// next one copied in (cp.async) while the current one is applied.  The 8 x 8 diagonal
+// systems take half a warp per column, real and imaginary part of a row in neighbouring
+// lanes: a step of their chain is two FP64 instructions, and of the lanes' work only half is
+// idle (blocks of 16 spent a quarter of the kernel there).  Bound by the FP64 pipe, n^2 CB
+// complex multiply-adds a CTA, and by the 2 n dependent steps when CB is small.
+constexpr int SP = 8;              // panel columns
+constexpr int SPL = SP + 1;
+size_t solve_smem(int n, int cb) { return sizeof(double2) * ((size_t)n * cb + 2 * (size_t)n * SPL + n); }
 
 template <bool GREEN>
 __global__ void __launch_bounds__(256) k_solve(SweepSys sys, const SweepJob* __restrict__ jobs, int i, int CB) {
@@ -419,13 +423,35 @@ __global__ void __launch_bounds__(256) k_solve(SweepSys sys, const SweepJob* __r
     const int first = last ? n : 0, end = n + y_cols(J, last, GREEN);   // X_{N-1} is not used
     const int c0 = first + blockIdx.x * CB, cb = min(CB, end - c0);
     if (cb <= 0) return;
-    constexpr int PL = solve_panel_ld();
     double2* X = sv;                        // n x CB
-    double2* F = sv + (size_t)n * CB;       // panel: rows x 16
-    const int t = threadIdx.x, lane = t & 31, hl = lane & 15, half = (t >> 5) * 2 + (lane >> 4);
+    double2* F = sv + (size_t)n * CB;       // two panels: rows x 8
+    double2* invd = F + 2 * (size_t)n * SPL;
+    const int t = threadIdx.x, hl = (t & 15) >> 1, part = t & 1, half = t >> 4;
     double2* R = J.XY + (size_t)i * n * w;
     const int* perm = perm_of(sys, J);
     const double2* HV1 = last ? nullptr : hv1_of(sys, J, i);
+    const double2* S = J.S;
+    const int nk = (n + SP - 1) / SP;
+    // panel step s = 0 .. 2 nk - 1: forward panels from the left, then backward from the right
+    auto geom = [&](int s, int& kb, int& ra, int& rows) {
+        const bool back = s >= nk;
+        kb = (back ? 2 * nk - 1 - s : s) * SP;
+        ra = back ? 0 : kb;
+        rows = (back ? min(kb + SP, n) : n) - ra;
+    };
+    auto copy = [&](int s) {
+        int kb, ra, rows;
+        geom(s, kb, ra, rows);
+        double2* dst = F + (size_t)(s & 1) * n * SPL;
+        for (int q = t; q < rows * SP; q += 256) {
+            const int r = q / SP, k = q % SP;
+            if (kb + k < n)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" :: "r"((uint32_t)__cvta_generic_to_shared(dst + r * SPL + k)),
+                             "l"(S + (size_t)(ra + r) * n + kb + k) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    copy(0);
     for (int q = t; q < n * cb; q += 256) {
         const int r = q / cb, c = c0 + q % cb, p = perm[r];
         double2 v;
@@ -439,59 +465,58 @@ __global__ void __launch_bounds__(256) k_solve(SweepSys sys, const SweepJob* __r
         }
         X[r * CB + q % cb] = v;
     }
-    const double2* S = J.S;
-    const int nk = (n + 15) / 16;
-    for (int pass = 0; pass < 2; ++pass)
-        for (int kk = 0; kk < nk; ++kk) {
-            const int kb = (pass ? nk - 1 - kk : kk) * 16, wd = min(16, n - kb);
-            const int ra = pass ? 0 : kb, rows = (pass ? kb + wd : n) - ra;     // panel rows [ra, ra + rows)
+    for (int r = t; r < n; r += 256) {
+        const double2 d = S[(size_t)r * n + r];
+        invd[r] = d.x == 0.0 && d.y == 0.0 ? make_double2(1, 0) : lu::inverse(d);
+    }
+    for (int s = 0; s < 2 * nk; ++s) {
+        int kb, ra, rows;
+        geom(s, kb, ra, rows);
+        const bool back = s >= nk;
+        const int wd = min(SP, n - kb);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();            // panel s landed, panel s - 1 applied
+        if (s + 1 < 2 * nk) copy(s + 1);
+        double2* P = F + (size_t)(s & 1) * n * SPL;
+        double2* D = P + (kb - ra) * SPL;             // diagonal block
+        if (back) {                 // its rows over their diagonal: a unit upper triangle
+            if (t < SP * SP && t / SP < wd && t % SP < wd) D[t / SP * SPL + t % SP] = cmul(D[t / SP * SPL + t % SP], invd[kb + t / SP]);
             __syncthreads();
-            for (int q = t; q < rows * 16; q += 256) {
-                const int r = q / 16, k = q % 16;
-                F[r * PL + k] = k < wd ? S[(size_t)(ra + r) * n + kb + k] : make_double2(0, 0);
-            }
-            __syncthreads();
-            const double2* D = F + (kb - ra) * PL;       // diagonal block
-            for (int cp = half; cp < ((cb + 15) / 16) * 16; cp += 16) {
-                const int c = min(cp, cb - 1);
-                double2 x = hl < wd ? X[(kb + hl) * CB + c] : make_double2(0, 0);
-                if (pass == 0) {
-                    for (int j = 0; j < wd - 1; ++j) {
-                        const double2 xj = make_double2(__shfl_sync(0xffffffffu, x.x, j, 16), __shfl_sync(0xffffffffu, x.y, j, 16));
-                        if (hl > j && hl < wd) x = lu::fnma(x, D[hl * PL + j], xj);
-                    }
-                } else {
-                    double2 d = hl < wd ? D[hl * PL + hl] : make_double2(1, 0);
-                    if (d.x == 0.0 && d.y == 0.0) d = make_double2(1, 0);
-                    const double2 inv = lu::inverse(d);
-                    for (int j = wd - 1; j >= 0; --j) {
-                        if (hl == j) x = cmul(x, inv);
-                        const double2 xj = make_double2(__shfl_sync(0xffffffffu, x.x, j, 16), __shfl_sync(0xffffffffu, x.y, j, 16));
-                        if (hl < j) x = lu::fnma(x, D[hl * PL + j], xj);
-                    }
-                }
-                if (hl < wd && cp < cb) X[(kb + hl) * CB + c] = x;
-            }
-            __syncthreads();
-            // the rows still to come minus panel x solved block
-            const int rb = pass ? 0 : kb + wd, re = pass ? kb : n;
-            for (int q = t; q < (re - rb) * cb; q += 256) {
-                const int r = rb + q / cb, c = q % cb;
-                const double2* f = F + (r - ra) * PL;
-                const double2* x = X + kb * CB + c;
-                double rr = 0, ii = 0, ri = 0, ir = 0;
-#pragma unroll 4
-                for (int k = 0; k < wd; ++k) {
-                    const double2 a = f[k], b = x[k * CB];
-                    rr = fma(a.x, b.x, rr);
-                    ii = fma(a.y, b.y, ii);
-                    ri = fma(a.x, b.y, ri);
-                    ir = fma(a.y, b.x, ir);
-                }
-                double2& v = X[r * CB + c];
-                v = make_double2(v.x - (rr - ii), v.y - (ri + ir));
-            }
         }
+        for (int cp = half; cp < (cb + 15) / 16 * 16; cp += 16) {
+            const int c = min(cp, cb - 1), row = min(kb + hl, n - 1);
+            const bool in = hl < wd && cp < cb;
+            double* xp = reinterpret_cast<double*>(X + row * CB + c) + part;
+            double x = *xp;
+            if (back) {
+                const double o = __shfl_xor_sync(0xffffffffu, x, 1);
+                const double2 v = invd[row];
+                x = part ? fma(x, v.x, o * v.y) : fma(x, v.x, -(o * v.y));
+            }
+            for (int q = 0; q < wd - 1; ++q) {
+                const int j = back ? wd - 1 - q : q;
+                const double xr = __shfl_sync(0xffffffffu, x, 2 * j, 16), xi = __shfl_sync(0xffffffffu, x, 2 * j + 1, 16);
+                if (in && (back ? hl < j : hl > j)) {
+                    const double2 d = D[hl * SPL + j];
+                    x = part ? fma(-d.x, xi, fma(-d.y, xr, x)) : fma(-d.x, xr, fma(d.y, xi, x));
+                }
+            }
+            if (in) *xp = x;
+        }
+        __syncthreads();
+        // the rows still to come minus panel x solved block
+        const int rb = back ? 0 : kb + wd, re = back ? kb : n;
+        for (int q = t; q < (re - rb) * cb; q += 256) {
+            const int r = rb + q / cb, c = q % cb;
+            const double2* f = P + (r - ra) * SPL;
+            const double2* x = X + kb * CB + c;
+            double2 v = X[r * CB + c];
+#pragma unroll
+            for (int k = 0; k < SP; ++k)
+                if (k < wd) v = lu::fnma(v, f[k], x[k * CB]);
+            X[r * CB + c] = v;
+        }
+    }
     __syncthreads();
     for (int q = t; q < n * cb; q += 256) R[(size_t)(q / cb) * w + c0 + q % cb] = X[(q / cb) * CB + q % cb];
 }
@@ -499,9 +524,10 @@ __global__ void __launch_bounds__(256) k_solve(SweepSys sys, const SweepJob* __r
 // ---------------------------------------------------------------- node back substitution
 // c_i = y_i - X_i c_{i+1} for columns [g0, g0 + CB) of one energy, i = N-2 .. 0 (c
 // overwrites y): the columns are independent, so a CTA carries its own through all nodes.
+// KS (a power of two) threads split an entry's sum where the entries alone leave threads idle.
 size_t back_smem(int n, int cb) { return sizeof(double2) * 2 * (size_t)n * cb; }
 
-__global__ void __launch_bounds__(256) k_back(SweepSys sys, const SweepJob* __restrict__ jobs, int CB) {
+__global__ void __launch_bounds__(256) k_back(SweepSys sys, const SweepJob* __restrict__ jobs, int CB, int KS) {
     extern __shared__ __align__(16) double2 sv[];
     const SweepJob& J = jobs[blockIdx.y];
     const int n = sys.n, N = sys.N, m = J.ms + J.md, w = n + m;
@@ -514,24 +540,24 @@ __global__ void __launch_bounds__(256) k_back(SweepSys sys, const SweepJob* __re
     for (int i = N - 2; i >= 0; --i) {
         double2* R = J.XY + (size_t)i * n * w;
         __syncthreads();
-        for (int q = t; q < n * cb; q += 256) {
-            const int r = q / cb, g = q % cb;
+        // KS neighbouring threads share an entry, each with every KS-th k
+        for (int q0 = 0; q0 < n * cb * KS; q0 += 256) {
+            const int q = min(q0 + t, n * cb * KS - 1) / KS, r = q / cb, g = q % cb;
             const double2* x = R + (size_t)r * w;
-            const double2* c = cur + g;
-            double rr = 0, ii = 0, ri = 0, ir = 0;
-#pragma unroll 8
-            for (int k = 0; k < n; ++k) {
-                const double2 a = x[k], b = c[k * cb];
-                rr = fma(a.x, b.x, rr);
-                ii = fma(a.y, b.y, ii);
-                ri = fma(a.x, b.y, ri);
-                ir = fma(a.y, b.x, ir);
+            double2 s = make_double2(0, 0);
+#pragma unroll 4
+            for (int k = t % KS; k < n; k += KS) cfma(s, x[k], cur[k * cb + g]);
+            for (int o = KS >> 1; o > 0; o >>= 1) {
+                s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+                s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
             }
-            double2& y = R[(size_t)r * w + n + g0 + g];
-            const double2 y0 = g0 + g < J.ms ? y : make_double2(0, 0);      // drain columns of y_i are zero
-            const double2 v = make_double2(y0.x - (rr - ii), y0.y - (ri + ir));
-            y = v;
-            nxt[q] = v;
+            if (t % KS == 0 && q0 + t < n * cb * KS) {
+                double2& y = R[(size_t)r * w + n + g0 + g];
+                const double2 y0 = g0 + g < J.ms ? y : make_double2(0, 0);      // drain columns of y_i are zero
+                const double2 v = csub(y0, s);
+                y = v;
+                nxt[q] = v;
+            }
         }
         double2* s = cur;
         cur = nxt;
@@ -553,13 +579,13 @@ __global__ void __launch_bounds__(256) k_green_product(SweepSys sys, const Sweep
     const double2 zero = make_double2(0, 0);
     double2 acc[R][R];
     if (stage == 0) {
-        tile_product<R>(sm, r0, c0, n, [&](int r, int k) { return r < n ? P[(size_t)r * w + k] : zero; },
+        tile_product<R>(sm, r0, c0, n, n, n, [&](int r, int k) { return r < n ? P[(size_t)r * w + k] : zero; },
                         [&](int k, int c) { return c < n ? Gn[(size_t)k * w + c] : zero; }, acc);
     } else if (stage == 1) {
         const double2* HV1 = hv1_of(sys, J, i);
         const double2* M1 = sys.M1;
         const double E = J.E;
-        tile_product<R>(sm, r0, c0, n,
+        tile_product<R>(sm, r0, c0, n, n, n,
                         [&](int r, int k) {
                             if (r >= n) return zero;
                             const size_t q = (size_t)k * n + r;
@@ -567,7 +593,7 @@ __global__ void __launch_bounds__(256) k_green_product(SweepSys sys, const Sweep
                         },
                         [&](int k, int c) { return c < n ? P[(size_t)k * w + n + c] : zero; }, acc);
     } else {
-        tile_product<R>(sm, r0, c0, n, [&](int r, int k) { return r < n ? J.S[(size_t)r * n + k] : zero; },
+        tile_product<R>(sm, r0, c0, n, n, n, [&](int r, int k) { return r < n ? J.S[(size_t)r * n + k] : zero; },
                         [&](int k, int c) { return c < n ? P[(size_t)k * w + c] : zero; }, acc);
     }
 #pragma unroll
@@ -617,7 +643,7 @@ __global__ void __launch_bounds__(256) k_residual_fp64(SweepSys sys, const ResJo
     };
     auto rhs = [&](const double2* c) { return [=](int k, int g) { return g < m ? c[(size_t)k * J.row_stride + g] : zero; }; };
     const double2* ci = J.C + (size_t)i * J.node_stride;
-    tile_product<R>(sm, r0, c0, n, [&](int r, int k) {
+    tile_product<R>(sm, r0, c0, n, m, n, [&](int r, int k) {
         if (r >= n) return zero;
         const size_t q = (size_t)r * n + k;
         double2 d = csub(cscale(M0[q], E), HV0[q]);
@@ -627,7 +653,7 @@ __global__ void __launch_bounds__(256) k_residual_fp64(SweepSys sys, const ResJo
     }, rhs(ci), acc);
     add();
     if (i + 1 < N) {
-        tile_product<R>(sm, r0, c0, n, [&](int r, int k) {
+        tile_product<R>(sm, r0, c0, n, m, n, [&](int r, int k) {
             if (r >= n) return zero;
             const size_t q = (size_t)r * n + k;
             return csub(cscale(M1[q], E), HV1[q]);
@@ -636,7 +662,7 @@ __global__ void __launch_bounds__(256) k_residual_fp64(SweepSys sys, const ResJo
     }
     if (i > 0) {
         const double2* HVm = HV1 - nn;
-        tile_product<R>(sm, r0, c0, n, [&](int r, int k) {
+        tile_product<R>(sm, r0, c0, n, m, n, [&](int r, int k) {
             if (r >= n) return zero;
             const size_t q = (size_t)k * n + r;
             return cconj(csub(cscale(M1[q], E), HVm[q]));
@@ -707,24 +733,14 @@ __global__ void __launch_bounds__(128) k_sweep_small(SweepSys sys, const SweepJo
     int bad = 0;
     // warp 0: best row of column c not used yet (n <= 32: a lane per row)
     auto search = [&](int c) {
-        double best = -2.0;
-        int idx = lane;
-        if (lane < n && step[lane] < 0) {
-            const double2 v = A[(size_t)lane * la + c];
-            best = fabs(v.x) + fabs(v.y);
-            if (!(best >= 0.0)) best = -1.0;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const double ov = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-            if (ov > best || (ov == best && oi < idx)) { best = ov; idx = oi; }
-        }
-        if (lane == 0) {
-            const double2 p = A[(size_t)idx * la + c];
-            const bool z = p.x == 0.0 && p.y == 0.0;
-            sel = idx;
+        const bool in = lane < n && step[lane] < 0;
+        const double2 p = in ? A[(size_t)lane * la + c] : make_double2(1, 0);
+        const bool z = p.x == 0.0 && p.y == 0.0;
+        const double2 inv = z ? make_double2(1, 0) : lu::inverse(p);       // every row's, beside the search
+        if (lu::warp_best(in ? lu::mag_key(fabs(p.x) + fabs(p.y)) : 0ull) == lane) {
+            sel = lane;
             szero = z;
-            sinv = z ? make_double2(1, 0) : lu::inverse(p);
+            sinv = inv;
         }
     };
     for (int i = 0; i < N; ++i) {
@@ -852,11 +868,11 @@ __global__ void __launch_bounds__(128) k_sweep_small(SweepSys sys, const SweepJo
 namespace {
 
 // columns per CTA so that `cols` columns of nb energies fill the SMs once, at most 32
-int column_block(int cols, int nb, int sms, size_t per_col, size_t fixed, int smem_max) {
+int column_block(int cols, int nb, int sms, size_t per_col, size_t fixed, int smem_max, int least) {
     const int fit = (int)std::min<size_t>(32, ((size_t)smem_max - fixed) / per_col);
     for (int waves = 1;; ++waves) {
         int cb = (int)(((long long)cols * nb + (long long)sms * waves - 1) / ((long long)sms * waves));
-        cb = std::max(cb, 4);
+        cb = std::max(cb, least);
         while (cb <= fit && (long long)((cols + cb - 1) / cb) * nb > (long long)sms * waves) ++cb;   // ragged blocks
         if (cb <= fit) return cb;
         if (waves > cols * nb) return fit;
@@ -885,7 +901,7 @@ int sweep_tiled(const SweepSys& sys, const SweepJob* jobs, const SweepJob* host,
         launches += 2;
         const int cols = (last ? 0 : n) + (GREEN ? n : yc);
         if (cols > 0) {
-            const int cb = column_block(cols, nb, sms, sizeof(double2) * n, solve_smem(n, 0), smem_max);
+            const int cb = column_block(cols, nb, sms, sizeof(double2) * n, solve_smem(n, 0), smem_max, 2);
             k_solve<GREEN><<<dim3((cols + cb - 1) / cb, nb), 256, solve_smem(n, cb), st>>>(sys, jobs, i, cb);
             ++launches;
         }
@@ -900,8 +916,10 @@ int sweep_tiled(const SweepSys& sys, const SweepJob* jobs, const SweepJob* host,
         k_green_dos<<<dim3(N, nb), 256, 0, st>>>(n, jobs);
         ++launches;
     } else if (m > 0) {
-        const int cb = column_block(m, nb, sms, 2 * sizeof(double2) * n, 0, smem_max);
-        k_back<<<dim3((m + cb - 1) / cb, nb), 256, back_smem(n, cb), st>>>(sys, jobs, cb);
+        const int cb = column_block(m, nb, sms, 2 * sizeof(double2) * n, 0, smem_max, 1);
+        int ks = 1;
+        while (ks < 16 && 2 * ks * n * cb <= 256) ks *= 2;
+        k_back<<<dim3((m + cb - 1) / cb, nb), 256, back_smem(n, cb), st>>>(sys, jobs, cb, ks);
         ++launches;
     }
     return launches;
@@ -934,7 +952,8 @@ int launch_sweep_fp64(const SweepSys& sys, const SweepJob* jobs, const SweepJob*
 void launch_residual_fp64(const SweepSys& sys, const ResJob* jobs, int m, int nb, cudaStream_t st) {
     if (m > 0) {
         const int t32 = (sys.n + 31) / 32, t16 = (sys.n + 15) / 16, c32 = (m + 31) / 32, c16 = (m + 15) / 16;
-        if ((long long)t32 * c32 * sys.N * nb >= 304) k_residual_fp64<2><<<dim3(sys.N, t32 * c32, nb), 256, 0, st>>>(sys, jobs);
+        // 32 x 32 tiles unless 16 x 16 ones cover the rows and columns with a tenth less
+        if (10ll * t16 * c16 >= 36ll * t32 * c32) k_residual_fp64<2><<<dim3(sys.N, t32 * c32, nb), 256, 0, st>>>(sys, jobs);
         else k_residual_fp64<1><<<dim3(sys.N, t16 * c16, nb), 256, 0, st>>>(sys, jobs);
     }
     launch_residual_finish(jobs, nb, st);
