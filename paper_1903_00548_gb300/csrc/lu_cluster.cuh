@@ -47,12 +47,14 @@ template <class T2> __device__ __forceinline__ T2 fnma(T2 a, T2 b, T2 c) {
 // |a|^2 well inside the range of normal numbers (by its exponent bits)
 __device__ __forceinline__ bool plain(double d) { const unsigned e = ((unsigned)__double2hiint(d) >> 20) & 0x7ff; return e - 64u < 1900u; }
 __device__ __forceinline__ bool plain(float d) { const unsigned e = (__float_as_uint(d) >> 23) & 0xff; return e - 10u < 230u; }
+__device__ __forceinline__ double recip(double d) { return 1.0 / d; }
+__device__ __forceinline__ float recip(float d) { return __frcp_rn(d); }
 // 1 / a; Smith's form where |a|^2 leaves that range
 template <class T2> __device__ __forceinline__ T2 inverse(T2 a) {
     using T = typename Real<T2>::t;
     const T d = fma(a.x, a.x, a.y * a.y);
     if (plain(d)) {
-        const T s = T(1) / d;
+        const T s = recip(d);
         return make2<T2>(a.x * s, -a.y * s);
     }
     if (fabs(a.x) >= fabs(a.y)) {

@@ -19,7 +19,7 @@ namespace pwqt {
 // CTAs per energy, a warp per out-mode with its lanes along the injected modes (one
 // energy's CTA took 0.6 ms at n = 128 and 77 modes when it did them alone).  The CTAs'
 // sums meet in the outputs, which the caller has zeroed.
-constexpr int OBS_CTAS = 16;
+constexpr int OBS_CTAS = 38;
 __global__ void __launch_bounds__(256) k_observables(int n, int N, const ObsJob* __restrict__ jobs) {
     const ObsJob& J = jobs[blockIdx.x];
     const int m = J.ms + J.md;
@@ -110,23 +110,28 @@ void launch_observables(int n, int N, const ObsJob* jobs, int nb, cudaStream_t s
 }
 
 // ---------------------------------------------------------------- residual
-__global__ void k_residual_finish(const ResJob* __restrict__ jobs, int nb, const int* __restrict__ active) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb || (active && !active[b])) return;
-    const ResJob J = jobs[b];
-    int m = J.ms + J.md;
+// a warp per energy (a thread walking the columns took 56 to 107 us at 55 to 93 of them)
+__global__ void __launch_bounds__(32) k_residual_finish(const ResJob* __restrict__ jobs, const int* __restrict__ active) {
+    const int b = blockIdx.x;
+    if (active && !active[b]) return;
+    const ResJob& J = jobs[b];
+    const int m = J.ms + J.md;
     double worst = 0.0;
-    for (int g = 0; g < m; ++g) {
-        double bb = J.bn2[g];
-        double v = bb > 0 ? sqrt(J.rn2[g] / bb) : sqrt(J.rn2[g]);
+    for (int g = threadIdx.x; g < m; g += 32) {
+        const double bb = J.bn2[g];
+        const double v = bb > 0 ? sqrt(J.rn2[g] / bb) : sqrt(J.rn2[g]);
         worst = (v > worst || isnan(v)) ? v : worst;   // NaN propagates (fmax would drop it)
         if (isnan(worst)) break;
     }
-    *J.resid = worst;
+    for (int o = 16; o > 0; o >>= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, worst, o);
+        worst = isnan(worst) ? worst : (v > worst || isnan(v)) ? v : worst;
+    }
+    if (threadIdx.x == 0) *J.resid = worst;
 }
 
 void launch_residual_finish(const ResJob* jobs, int nb, cudaStream_t st, const int* active) {
-    k_residual_finish<<<(nb + 127) / 128, 128, 0, st>>>(jobs, nb, active);
+    k_residual_finish<<<nb, 32, 0, st>>>(jobs, active);
 }
 
 __global__ void k_fill_int(int* p, int v, int cnt) {

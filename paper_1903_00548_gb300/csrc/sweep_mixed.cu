@@ -23,6 +23,7 @@
 
 #include "cgemm_tc.cuh"
 #include "residual_oz.cuh"
+#include "sweep_c64.cuh"
 #include "sweep_mixed.cuh"
 
 namespace pwqt {
@@ -981,11 +982,20 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
     int* active_d = (int*)take(sizeof(int) * nb);
     int* bits_d = (int*)take(sizeof(int) * nb);
 
-    // ---------------- forward sweep over the nodes
-    const int fblocks = (int)std::min<size_t>(((size_t)n * n + NT - 1) / NT, 512);
-    const size_t panel_smem = sizeof(float2) * (size_t)(n + 1) * PW;
+    // ---------------- forward sweep over the nodes, node back substitution
     int smem_optin = 0;
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->dev);
+    // up to block 320 a small cluster's shared memory holds the node block and the FP32 pipes
+    // beat the tensor-core form: three launches a node against 5 n / 32 (sweep of 16 energies
+    // at n = 128, 50 nodes: 57 -> 13 ms)
+    const bool small = c64_sweep_fits(n, smem_optin);
+    if (c->profile) PWQT_CUDA(c, cudaEventRecord(L.ev[0], st));
+    if (small) {
+        const C64Sweep cs{sys, jobs_d, m, w, S.F, S.sF, S.piv, S.sP, S.XY, S.sXY, S.Lb, S.sL, S.C64, S.sC};
+        c->launches += c64_sweep(cs, jobs.data(), nb, c->sm_count, smem_optin, st);
+    } else {
+    const int fblocks = (int)std::min<size_t>(((size_t)n * n + NT - 1) / NT, 512);
+    const size_t panel_smem = sizeof(float2) * (size_t)(n + 1) * PW;
     if (panel_smem > (size_t)smem_optin)
         return fail(c, PWQT_ERR_INVALID_ARG, "the complex64 panel of block size " + std::to_string(n) +
                                                  " exceeds shared memory: use PWQT_FP64 (mixed precision takes n <= " +
@@ -1005,7 +1015,6 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
         launch_cgemm_tc(g, nb, M, Nc, K, st);
         c->launches++;
     };
-    if (c->profile) PWQT_CUDA(c, cudaEventRecord(L.ev[0], st));
     for (int i = 0; i < N; ++i) {
         float2* Fi = S.F + (size_t)i * n * n;
         float2* XYi = S.XY + (size_t)i * n * w;
@@ -1040,6 +1049,7 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
         const float2* XYn = S.XY + (size_t)(i + 1) * n * w;
         gemm(XYi, S.sXY, w, XYn + n, S.sXY, w, XYn + n, S.sXY, w, XYi + n, S.sXY, w, XYi + n, S.sXY, w, m, n, m, n);
     }
+    }
     if (c->profile) {
         PWQT_CUDA(c, cudaEventRecord(L.ev[1], st));
         PWQT_CUDA(c, cudaEventSynchronize(L.ev[1]));
@@ -1051,10 +1061,13 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
     }
     PWQT_CUDA(c, cudaGetLastError());
     if (cgemm_tc_error(true, st)) return fail(c, PWQT_ERR_TIMEOUT, "tensor-core GEMM: a bounded mbarrier wait gave up");
-    k_mx_to64<<<dim3(256, nb), NT, 0, st>>>(S);
-    k_mx_perm<<<dim3(nb, N), 32, 2 * sizeof(int) * n, st>>>(S);
+    if (!small) {
+        k_mx_to64<<<dim3(256, nb), NT, 0, st>>>(S);
+        k_mx_perm<<<dim3(nb, N), 32, 2 * sizeof(int) * n, st>>>(S);
+        c->launches += 2;
+    }
     k_mx_diag_inv<<<dim3((n + TS - 1) / TS, N, nb), 32, 0, st>>>(S);
-    c->launches += 3;
+    c->launches++;
 
     // ---------------- refinement with FP64 residuals
     for (int b = 0; b < nb; ++b) {
