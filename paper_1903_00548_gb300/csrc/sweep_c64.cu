@@ -138,16 +138,27 @@ __global__ void __launch_bounds__(256) k_c64_node(C64Sweep S, int i) {
 
 // ---------------------------------------------------------------- solve for [X_i | y_i]
 // Columns [c0, c0 + CB) of P [U_i | y] through L and U, in shared memory; the factors in
-// panels of 16 columns, the next one copied in while the current one is applied.  Diagonal
+// panels of 16 columns, the next ones copied in while the current one is applied.  Diagonal
 // 16 x 16 systems: half a warp per column, a lane per row.  The update gives a thread four
 // rows of one column (two k of four factor rows per 16-byte load).
 constexpr int SP = 16;
 constexpr int SPL = SP + 2;        // rows on 16-byte boundaries
-size_t solve_smem(int n, int cb) { return sizeof(float2) * (2 * (size_t)n * SPL + (size_t)n * cb + n); }
+// shared memory with ns panels in flight
+size_t solve_smem(int n, int cb, int ns) { return sizeof(float2) * (ns * (size_t)n * SPL + (size_t)n * cb + n); }
 
-__device__ __forceinline__ void copy8(float2* dst, const float2* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+// rows of 16 factors (zero past column n, n even) to a panel buffer, 16 bytes at a time
+__device__ __forceinline__ void copy_panel(float2* dst, const float2* src, size_t ld, int rows, int kb, int n) {
+    for (int q = threadIdx.x; q < rows * (SP / 2); q += 256) {
+        const int r = q / (SP / 2), k = q % (SP / 2) * 2;
+        float2* d = dst + r * SPL + k;
+        if (kb + k < n)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"((uint32_t)__cvta_generic_to_shared(d)), "l"(src + r * ld + kb + k) : "memory");
+        else *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 }
+__device__ __forceinline__ void commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the newest K groups have landed
+template <int K> __device__ __forceinline__ void wait_groups() { asm volatile("cp.async.wait_group %0;" :: "n"(K) : "memory"); }
 
 // rows r .. r+3 (those below `re`) of column c: X -= panel rows (P + (r - ra) SPL) x solved block xb
 __device__ __forceinline__ void solve_rows(float2* X, int CB, const float2* P, const float2* xb, int r, int re) {
@@ -174,6 +185,59 @@ __device__ __forceinline__ void solve_rows(float2* X, int CB, const float2* P, c
         if (r + x < re) X[x * CB] = v[x];
 }
 
+// 16 x 16 diagonal systems of up to two columns, a lane (hl) per row: D is the lane's row of
+// the block (columns past wd zero), iv the reciprocal of its diagonal; unit lower or (back)
+// upper.  The two chains run side by side: a step is latency (two shuffles, two FMAs).
+__device__ __forceinline__ void diagonal(float2 (&x)[2], const float2* D, float2 iv, int hl, int wd, bool back) {
+    float2 d[SP];
+#pragma unroll
+    for (int j = 0; j < SP; j += 2) {
+        const float4 f = *reinterpret_cast<const float4*>(D + j);
+        d[j] = make_float2(f.x, f.y);
+        d[j + 1] = make_float2(f.z, f.w);
+    }
+    if (!back) {
+#pragma unroll
+        for (int j = 0; j < SP - 1; ++j)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const float2 xj = make_float2(__shfl_sync(0xffffffffu, x[c].x, j, 16), __shfl_sync(0xffffffffu, x[c].y, j, 16));
+                const float2 y = lu::fnma(x[c], d[j], xj);
+                x[c] = hl > j ? y : x[c];
+            }
+    } else {
+#pragma unroll
+        for (int j = SP - 1; j >= 0; --j)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const float2 z = lu::mul(x[c], iv);
+                x[c] = hl == j ? z : x[c];
+                const float2 xj = make_float2(__shfl_sync(0xffffffffu, x[c].x, j, 16), __shfl_sync(0xffffffffu, x[c].y, j, 16));
+                const float2 y = lu::fnma(x[c], d[j], xj);
+                x[c] = hl < j && j < wd ? y : x[c];
+            }
+    }
+}
+
+// rows [rb, re) of the columns minus panel x solved block (rows kb .. kb + wd)
+__device__ __forceinline__ void panel_update(float2* X, int CB, int cb, const float2* P, int ra, int kb, int wd, int rb, int re) {
+    const int t = threadIdx.x;
+    if (wd == SP) {
+        for (int q = t; q < (re - rb + 3) / 4 * cb; q += 256) {
+            const int r = rb + q / cb * 4, c = q % cb;
+            solve_rows(X + r * CB + c, CB, P + (r - ra) * SPL, X + kb * CB + c, r, re);
+        }
+    } else {                        // the ragged last block
+        for (int q = t; q < (re - rb) * cb; q += 256) {
+            const int r = rb + q / cb, c = q % cb;
+            float2 v = X[r * CB + c];
+            for (int k = 0; k < wd; ++k) v = lu::fnma(v, P[(r - ra) * SPL + k], X[(kb + k) * CB + c]);
+            X[r * CB + c] = v;
+        }
+    }
+}
+
+template <int NS>
 __global__ void __launch_bounds__(256) k_c64_solve(C64Sweep S, int i, int CB) {
     extern __shared__ __align__(16) float2 fsm[];
     const int e = blockIdx.y;
@@ -183,8 +247,8 @@ __global__ void __launch_bounds__(256) k_c64_solve(C64Sweep S, int i, int CB) {
     const int first = last ? n : 0, end = n + (last ? J.ms + J.md : J.ms);     // X_{N-1} is not used
     const int c0 = first + blockIdx.x * CB, cb = min(CB, end - c0);
     if (cb <= 0) return;
-    float2* F0 = fsm;                           // two panels of n x 16
-    float2* X = fsm + 2 * (size_t)n * SPL;      // n x CB (block rows past n are read from the last row)
+    float2* F0 = fsm;                           // NS panels of n x 16
+    float2* X = fsm + NS * (size_t)n * SPL;     // n x CB (block rows past n are read from the last row)
     float2* invd = X + (size_t)n * CB;
     const int t = threadIdx.x, hl = t & 15, half = t >> 4;
     float2* XYi = S.XY + e * S.sXY + (size_t)i * n * w;
@@ -199,17 +263,15 @@ __global__ void __launch_bounds__(256) k_c64_solve(C64Sweep S, int i, int CB) {
         rows = (back ? min(kb + SP, n) : n) - ra;
     };
     auto copy = [&](int s) {
-        int kb, ra, rows;
-        geom(s, kb, ra, rows);
-        float2* dst = F0 + (size_t)(s & 1) * n * SPL;
-        for (int q = t; q < rows * SP; q += 256) {
-            const int r = q / SP, k = q % SP;
-            if (kb + k < n) copy8(dst + r * SPL + k, F + (size_t)(ra + r) * n + kb + k);
-            else dst[r * SPL + k] = make_float2(0.f, 0.f);
+        if (s < 2 * nk) {
+            int kb, ra, rows;
+            geom(s, kb, ra, rows);
+            copy_panel(F0 + (size_t)(s % NS) * n * SPL, F + (size_t)ra * n, n, rows, kb, n);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        commit();
     };
-    copy(0);
+#pragma unroll
+    for (int s = 0; s < NS - 1; ++s) copy(s);
     for (int q = t; q < n * cb; q += 256) {
         const int r = q / cb, c = c0 + q % cb, p = perm[r];
         const size_t u = (size_t)p * n + c;
@@ -224,55 +286,20 @@ __global__ void __launch_bounds__(256) k_c64_solve(C64Sweep S, int i, int CB) {
         geom(s, kb, ra, rows);
         const bool back = s >= nk;
         const int wd = min(SP, n - kb);
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        wait_groups<NS - 2>();
         __syncthreads();            // panel s landed, panel s - 1 applied
-        if (s + 1 < 2 * nk) copy(s + 1);
-        const float2* P = F0 + (size_t)(s & 1) * n * SPL;
+        copy(s + NS - 1);
+        const float2* P = F0 + (size_t)(s % NS) * n * SPL;
         const float2* D = P + (kb - ra) * SPL;
-        for (int cp = half; cp < (cb + 15) / 16 * 16; cp += 16) {
-            const int c = min(cp, cb - 1), row = min(kb + hl, n - 1);
-            const bool in = hl < wd && cp < cb;
-            float2 x = X[row * CB + c];
-            const float2 iv = invd[row];
-            float2 d[SP];               // this lane's row of the block
-#pragma unroll
-            for (int j = 0; j < SP; j += 2) {
-                const float4 f = *reinterpret_cast<const float4*>(D + min(hl, wd - 1) * SPL + j);
-                d[j] = make_float2(f.x, f.y);
-                d[j + 1] = make_float2(f.z, f.w);
-            }
-            if (!back) {
-#pragma unroll
-                for (int j = 0; j < SP - 1; ++j) {
-                    const float2 xj = make_float2(__shfl_sync(0xffffffffu, x.x, j, 16), __shfl_sync(0xffffffffu, x.y, j, 16));
-                    if (hl > j) x = lu::fnma(x, d[j], xj);
-                }
-            } else {
-#pragma unroll
-                for (int j = SP - 1; j >= 0; --j) {
-                    if (hl == j) x = lu::mul(x, iv);
-                    const float2 xj = make_float2(__shfl_sync(0xffffffffu, x.x, j, 16), __shfl_sync(0xffffffffu, x.y, j, 16));
-                    if (hl < j && j < wd) x = lu::fnma(x, d[j], xj);
-                }
-            }
-            if (in) X[row * CB + c] = x;
+        for (int cp = half; cp < (cb + 15) / 16 * 16; cp += 32) {
+            const int c = min(cp, cb - 1), c2 = min(cp + 16, cb - 1), row = min(kb + hl, n - 1);
+            float2 x[2] = {X[row * CB + c], X[row * CB + c2]};
+            diagonal(x, D + min(hl, wd - 1) * SPL, invd[row], hl, wd, back);
+            if (hl < wd && cp < cb) X[row * CB + c] = x[0];
+            if (hl < wd && cp + 16 < cb) X[row * CB + c2] = x[1];
         }
         __syncthreads();
-        // the rows still to come minus panel x solved block
-        const int rb = back ? 0 : kb + wd, re = back ? kb : n, groups = (re - rb + 3) / 4;
-        if (wd == SP) {
-            for (int q = t; q < groups * cb; q += 256) {
-                const int r = rb + q / cb * 4, c = q % cb;
-                solve_rows(X + r * CB + c, CB, P + (r - ra) * SPL, X + kb * CB + c, r, re);
-            }
-        } else {                        // the ragged last block
-            for (int q = t; q < (re - rb) * cb; q += 256) {
-                const int r = rb + q / cb, c = q % cb;
-                float2 v = X[r * CB + c];
-                for (int k = 0; k < wd; ++k) v = lu::fnma(v, P[(r - ra) * SPL + k], X[(kb + k) * CB + c]);
-                X[r * CB + c] = v;
-            }
-        }
+        panel_update(X, CB, cb, P, ra, kb, wd, back ? 0 : kb + wd, back ? kb : n);
     }
     __syncthreads();
     for (int q = t; q < n * cb; q += 256) XYi[(size_t)(q / cb) * w + c0 + q % cb] = X[(q / cb) * CB + q % cb];
@@ -281,11 +308,12 @@ __global__ void __launch_bounds__(256) k_c64_solve(C64Sweep S, int i, int CB) {
 // ---------------------------------------------------------------- node back substitution
 // c_i = y_i - X_i c_{i+1}, i = N-2 .. 0, for columns [g0, g0 + CB) of one energy through all
 // nodes, written as FP64 (columns past the energy's own: zero).  X_i passes through shared
-// memory in panels of 16 columns, two in flight; a thread keeps up to BI groups of four rows
+// memory in panels of 16 columns, NS in flight; a thread keeps up to BI groups of four rows
 // of one column in registers.
 constexpr int BI = 4;
-size_t back_smem(int n, int cb) { return sizeof(float2) * (2 * (size_t)n * SPL + 2 * (size_t)(n + SP) * cb); }
+size_t back_smem(int n, int cb, int ns) { return sizeof(float2) * (ns * (size_t)n * SPL + 2 * (size_t)(n + SP) * cb); }
 
+template <int NS>
 __global__ void __launch_bounds__(256) k_c64_back(C64Sweep S, int CB) {
     extern __shared__ __align__(16) float2 fsm[];
     const int e = blockIdx.y;
@@ -294,24 +322,17 @@ __global__ void __launch_bounds__(256) k_c64_back(C64Sweep S, int CB) {
     const int g0 = blockIdx.x * CB, cb = min(CB, m - g0);
     if (cb <= 0) return;
     float2* F0 = fsm;
-    float2* cur = fsm + 2 * (size_t)n * SPL;          // rows n .. n + 15: zero
+    float2* cur = fsm + NS * (size_t)n * SPL;          // rows n .. n + 15: zero
     float2* nxt = cur + (size_t)(n + SP) * CB;
     const int t = threadIdx.x, nk = (n + SP - 1) / SP, groups = (n + 3) / 4;
     const float2* XY = S.XY + e * S.sXY;
     double2* Cd = S.C64 + e * S.sC;
     auto copy = [&](int s) {                           // panel s counts over all nodes, N-2 first
-        const int i = N - 2 - s / nk, kb = s % nk * SP;
-        const float2* X = XY + (size_t)i * n * w;
-        float2* dst = F0 + (size_t)(s & 1) * n * SPL;
-        for (int q = t; q < n * SP; q += 256) {
-            const int r = q / SP, k = q % SP;
-            if (kb + k < n) copy8(dst + r * SPL + k, X + (size_t)r * w + kb + k);
-            else dst[r * SPL + k] = make_float2(0.f, 0.f);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (s < (N - 1) * nk) copy_panel(F0 + (size_t)(s % NS) * n * SPL, XY + (size_t)(N - 2 - s / nk) * n * w, w, n, s % nk * SP, n);
+        commit();
     };
-    const int total = (N - 1) * nk;
-    if (total > 0) copy(0);
+#pragma unroll
+    for (int s = 0; s < NS - 1; ++s) copy(s);
     for (int q = t; q < 2 * (n + SP) * CB; q += 256) cur[q] = make_float2(0.f, 0.f);
     __syncthreads();
     for (int q = t; q < n * cb; q += 256) {
@@ -331,10 +352,10 @@ __global__ void __launch_bounds__(256) k_c64_back(C64Sweep S, int CB) {
         }
         for (int k = 0; k < nk; ++k) {
             const int s = (N - 2 - i) * nk + k;
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            wait_groups<NS - 2>();
             __syncthreads();
-            if (s + 1 < total) copy(s + 1);
-            const float2* P = F0 + (size_t)(s & 1) * n * SPL;
+            copy(s + NS - 1);
+            const float2* P = F0 + (size_t)(s % NS) * n * SPL;
 #pragma unroll
             for (int b = 0; b < BI; ++b) {
                 const int q = t + b * 256;
@@ -375,18 +396,23 @@ __global__ void __launch_bounds__(256) k_c64_back(C64Sweep S, int CB) {
 
 // columns per CTA so that `cols` columns of nb energies fill the SMs once (or, where `most`
 // forbids it, a whole number of times)
-int column_block(int cols, int nb, int sms, int most) {
+int column_block(int cols, int nb, int sms, int most, int least) {
     for (int waves = 1;; ++waves) {
         int cb = (int)(((long long)cols * nb + (long long)sms * waves - 1) / ((long long)sms * waves));
-        cb = std::max(cb, 4);
+        cb = std::max(cb, least);
         while (cb <= most && (long long)((cols + cb - 1) / cb) * nb > (long long)sms * waves) ++cb;
         if (cb <= most || waves > cols * nb) return std::min(cb, most);
     }
 }
+// panels in flight: 4 where four CTAs of that size share an SM, else 2 (the two halves of a
+// batch run side by side: at n = 128 four panels leave room for two CTAs, which cost 2 % of
+// the whole call)
+template <class Smem> int stages(int n, int cb, int smem_max, Smem smem) { return 4 * smem(n, cb, 4) <= (size_t)smem_max ? 4 : 2; }
+template <class F> void allow_smem(F* f, int smem_max) { cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max); }
 }  // namespace
 
 bool c64_sweep_fits(int n, int smem_max) {
-    return n > 24 && lup::pick_cluster(n, smem_max) > 0 && solve_smem(n, 8) <= (size_t)smem_max && back_smem(n, 8) <= (size_t)smem_max;
+    return n > 24 && lup::pick_cluster(n, smem_max) > 0 && solve_smem(n, 8, 2) <= (size_t)smem_max && back_smem(n, 8, 2) <= (size_t)smem_max;
 }
 
 int c64_sweep(const C64Sweep& S, const SweepJob* host, int nb, int sms, int smem_max, cudaStream_t st) {
@@ -394,14 +420,16 @@ int c64_sweep(const C64Sweep& S, const SweepJob* host, int nb, int sms, int smem
     int ms = 0, launches = 0;
     for (int b = 0; b < nb; ++b) ms = std::max(ms, host[b].ms);
     const int C = lup::pick_cluster(n, smem_max);
-    cudaFuncSetAttribute(k_c64_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-    cudaFuncSetAttribute(k_c64_back, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    allow_smem(k_c64_solve<2>, smem_max);
+    allow_smem(k_c64_solve<4>, smem_max);
+    allow_smem(k_c64_back<2>, smem_max);
+    allow_smem(k_c64_back<4>, smem_max);
     // 64 x 64 tiles once they give every other SM a CTA (two halves of a batch share the chip)
     const int t32 = (n + 31) / 32, t64 = (n + 63) / 64;
     const bool big = (long long)t64 * t64 * nb * 2 >= sms;
     k_c64_couplings<<<dim3(N - 1, t32 * t32, nb), 256, 0, st>>>(S);
     ++launches;
-    const int most_s = (int)std::min<size_t>(64, ((size_t)smem_max - solve_smem(n, 0)) / (sizeof(float2) * n));
+    const int most_s = (int)std::min<size_t>(64, ((size_t)smem_max - solve_smem(n, 0, 2)) / (sizeof(float2) * n));
     for (int i = 0; i < N; ++i) {
         const bool last = i == N - 1;
         const int yc = last ? S.m : ms;
@@ -412,15 +440,21 @@ int c64_sweep(const C64Sweep& S, const SweepJob* host, int nb, int sms, int smem
         launches += 2;
         const int cols = (last ? 0 : n) + yc;
         if (cols > 0) {
-            const int cb = column_block(cols, nb, sms, most_s);
-            k_c64_solve<<<dim3((cols + cb - 1) / cb, nb), 256, solve_smem(n, cb), st>>>(S, i, cb);
+            const int cb = column_block(cols, nb, sms, most_s, 4);
+            const int ns = stages(n, cb, smem_max, solve_smem);
+            const dim3 grid((cols + cb - 1) / cb, nb);
+            if (ns == 4) k_c64_solve<4><<<grid, 256, solve_smem(n, cb, 4), st>>>(S, i, cb);
+            else k_c64_solve<2><<<grid, 256, solve_smem(n, cb, 2), st>>>(S, i, cb);
             ++launches;
         }
     }
     const int groups = (n + 3) / 4;
-    const int most_b = (int)std::min<size_t>(256 * BI / groups, ((size_t)smem_max - back_smem(n, 0)) / (2 * sizeof(float2) * (n + SP)));
-    const int cb = column_block(S.m, nb, sms, most_b);
-    k_c64_back<<<dim3((S.m + cb - 1) / cb, nb), 256, back_smem(n, cb), st>>>(S, cb);
+    const int most_b = (int)std::min<size_t>(256 * BI / groups, ((size_t)smem_max - back_smem(n, 0, 2)) / (2 * sizeof(float2) * (n + SP)));
+    const int cb = column_block(S.m, nb, sms, most_b, 4);
+    const int ns = stages(n, cb, smem_max, back_smem);
+    const dim3 grid((S.m + cb - 1) / cb, nb);
+    if (ns == 4) k_c64_back<4><<<grid, 256, back_smem(n, cb, 4), st>>>(S, cb);
+    else k_c64_back<2><<<grid, 256, back_smem(n, cb, 2), st>>>(S, cb);
     return launches + 1;
 }
 
