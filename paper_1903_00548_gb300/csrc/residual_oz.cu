@@ -24,7 +24,7 @@
 //     B'[s]    = [ Re c_j ; Im c_j ]  (j = node of segment s),
 // so (A'B')[2r] = Re (A c)_r and (A'B')[2r+1] = Im (A c)_r.
 //
-// Kernel.  One CTA per (item, 128-row tile, 32-column tile); an item is a node (M
+// Kernel.  A tile is (item, 128 rows, 32 columns); an item is a node (M
 // and HV products) or an (energy, contact) pair (Sigma products).  Operand tiles are
 // stored pre-packed in the UMMA canonical K-major layout (8 rows x 16 bytes core
 // matrices), one contiguous block per 32-K chunk and slice, and moved by 1D bulk
@@ -302,46 +302,49 @@ __global__ void k_c_slice(const double2* __restrict__ C, long long sC, const int
 }
 
 // ---------------------------------------------------------------- the slice-product GEMM
-__global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const GemmArgs G) {
+// One output tile of a launch.  Segments present are a contiguous range [s_lo, s_lo + nseg)
+// of the item's segments; segment s reads the solution of node node0 + s.
+struct Tile {
+    int ct, rt, node, e_act, aitem, nseg_tot, s_lo, nseg, node0;
+};
+
+// Tile q of the launch (columns fastest, then rows, then items); false: nothing to compute.
+// Item z: node z with segments j = z-1, z, z+1 (M, HV), or the contact's edge node of active
+// energy z with one segment (Sigma).  Launches over one energy or one system's energies
+// start at the first column tile of their range.
+__device__ __forceinline__ bool tile_of(const GemmArgs& G, int q, int ctiles, Tile& T) {
+    const int RT = 2 * G.n_pad / TM, z = q / (ctiles * RT);
+    T.rt = q / ctiles % RT;
+    T.ct = q % ctiles + (G.mode == MODE_SIGMA ? z * G.m : G.col_lo) / TN;
+    T.e_act = -1;
+    if (G.mode == MODE_SIGMA) {
+        T.e_act = z;
+        T.node = T.node0 = G.sigma_side ? G.N - 1 : 0;
+        T.nseg_tot = T.nseg = 1;
+        T.s_lo = 0;
+        if (z >= G.n_act) return false;
+        T.aitem = 2 * G.act[z] + G.sigma_side;
+        return T.ct * TN < z * G.m + G.m && T.ct * TN + TN > z * G.m;      // columns of that energy only
+    }
+    T.node = z;
+    T.nseg_tot = 3;
+    T.s_lo = z == 0 ? 1 : 0;
+    T.nseg = (z == G.N - 1 ? 1 : 2) - T.s_lo + 1;
+    T.node0 = z - 1;
+    T.aitem = G.mode == MODE_M ? 0 : z;
+    return T.ct < G.nct && T.ct * TN < G.col_hi && T.ct * TN + TN > G.col_lo;
+}
+
+// Persistent: one CTA per SM walks the launch's tiles (q = block, block + grid, ...), the
+// chunk and stage counters running on, so that barriers, tensor memory and the zero slices
+// are set up once and the producer and the MMAs are in the next tile while the drain warps
+// write the last one (a CTA per tile spent more than half of its time at its two ends where
+// K is short: 38 us a tile at n = 128 for 14 us of MMAs).
+__global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const GemmArgs G, int ctiles, int ntiles) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    // column tile: launches over one energy (Sigma) or one system's energies (HV) start at
-    // the first tile of their column range
-    const int c_first = G.mode == MODE_SIGMA ? (int)blockIdx.z * G.m : G.col_lo;
-    const int ct = blockIdx.x + c_first / TN, rt = blockIdx.y, z = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n = G.n, N = G.N, m = G.m, n_pad = G.n_pad;
-    const int RT = 2 * n_pad / TM, KC = 2 * n_pad / KCH;
-
-    // ---- the item: node and segments (M, HV: node z, segments j = z-1, z, z+1; Sigma:
-    // item z = 2 k + side of active energy k, one segment at the contact's edge node)
-    // segments present are a contiguous range [s_lo, s_lo + nseg) of the item's
-    // segments; segment s reads the solution of node node0 + s
-    int node, e_act = -1, aitem, nseg_tot, s_lo, nseg, node0;
-    if (G.mode == MODE_SIGMA) {
-        e_act = z;
-        if (e_act >= G.n_act) return;
-        node = G.sigma_side ? N - 1 : 0;
-        nseg_tot = 1;
-        s_lo = 0;
-        nseg = 1;
-        node0 = node;
-        aitem = 2 * G.act[e_act] + G.sigma_side;
-        // columns of that energy only
-        const int c_lo = e_act * m, c_hi = c_lo + m;
-        if (ct * TN >= c_hi || ct * TN + TN <= c_lo) return;
-    } else {
-        if (ct >= G.nct || ct * TN >= G.col_hi || ct * TN + TN <= G.col_lo) return;
-        node = z;
-        nseg_tot = 3;
-        s_lo = node == 0 ? 1 : 0;
-        const int s_hi = node == N - 1 ? 1 : 2;
-        nseg = s_hi - s_lo + 1;
-        node0 = node - 1;
-        aitem = G.mode == MODE_M ? 0 : z;
-    }
-    (void)RT;
-    const int nchunks = nseg * KC;
-    const int nstages = nchunks / KSTAGE_CHUNKS;
+    const int KC = 2 * n_pad / KCH;
 
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + NSTAGE * STAGE_BYTES);
     // full[3] | empty[3] | accfull[2] | accempty[2] | tmem slot | abort flag
@@ -377,44 +380,54 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const GemmArgs G) {
     if (warp == 0) {
         // ---------------- producer
         if (lane == 0) {
-            const char* Abase = reinterpret_cast<const char*>(G.A) + (size_t)aitem * G.a_item_bytes;
-            for (int c = 0; c < nchunks; ++c) {
-                const int st = c % NSTAGE;
-                if (c >= NSTAGE && !mbar_wait(empty0 + 8 * st, ((c / NSTAGE) - 1) & 1)) { *abort_flag = 1; break; }
-                if (*abort_flag) break;
-                const int s = s_lo + c / KC, kc = c % KC, j = node0 + s;
-                const char* a = Abase + ((((size_t)rt * nseg_tot + s) * KC + kc) * A_CHUNK_BYTES);
-                const char* b = reinterpret_cast<const char*>(G.B) + ((((size_t)j * G.nct + ct) * KC + kc) * B_CHUNK_BYTES);
-                const uint32_t dst = smem0 + st * STAGE_BYTES;
-                mbar_expect_tx(full0 + 8 * st, A_CHUNK_BYTES + B_CHUNK_BYTES);
-                bulk_g2s(dst, a, A_CHUNK_BYTES, full0 + 8 * st);
-                bulk_g2s(dst + A_CHUNK_BYTES, b, B_CHUNK_BYTES, full0 + 8 * st);
-                issued = c + 1;
+            bool go = true;
+            for (int q = blockIdx.x; q < ntiles && go; q += gridDim.x) {
+                Tile T;
+                if (!tile_of(G, q, ctiles, T)) continue;
+                const char* Abase = reinterpret_cast<const char*>(G.A) + (size_t)T.aitem * G.a_item_bytes;
+                for (int c = 0; c < T.nseg * KC; ++c) {
+                    const int g = issued, st = g % NSTAGE;
+                    if (g >= NSTAGE && !mbar_wait(empty0 + 8 * st, ((g / NSTAGE) - 1) & 1)) { *abort_flag = 1; go = false; break; }
+                    if (*abort_flag) { go = false; break; }
+                    const int s = T.s_lo + c / KC, kc = c % KC, j = T.node0 + s;
+                    const char* a = Abase + ((((size_t)T.rt * T.nseg_tot + s) * KC + kc) * A_CHUNK_BYTES);
+                    const char* b = reinterpret_cast<const char*>(G.B) + ((((size_t)j * G.nct + T.ct) * KC + kc) * B_CHUNK_BYTES);
+                    const uint32_t dst = smem0 + st * STAGE_BYTES;
+                    mbar_expect_tx(full0 + 8 * st, A_CHUNK_BYTES + B_CHUNK_BYTES);
+                    bulk_g2s(dst, a, A_CHUNK_BYTES, full0 + 8 * st);
+                    bulk_g2s(dst + A_CHUNK_BYTES, b, B_CHUNK_BYTES, full0 + 8 * st);
+                    issued = g + 1;
+                }
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer
         if (lane == 0) {
-            for (int c = 0; c < nchunks; ++c) {
-                const int st = c % NSTAGE, ps = c / KSTAGE_CHUNKS, buf = ps & 1;
-                if (c % KSTAGE_CHUNKS == 0 && ps >= 2 && !mbar_wait(acce0 + 8 * buf, ((ps >> 1) - 1) & 1)) { *abort_flag = 1; break; }
-                if (!mbar_wait(full0 + 8 * st, (c / NSTAGE) & 1)) { *abort_flag = 1; break; }
-                if (*abort_flag) break;
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const uint32_t a0 = smem0 + st * STAGE_BYTES, b0 = a0 + A_CHUNK_BYTES;
-                const uint32_t d0 = tmem + (uint32_t)buf * ACC_COLS;
+            bool go = true;
+            for (int q = blockIdx.x; q < ntiles && go; q += gridDim.x) {
+                Tile T;
+                if (!tile_of(G, q, ctiles, T)) continue;
+                for (int c = 0; c < T.nseg * KC; ++c) {      // whole accumulation stages per tile
+                    const int g = mma_chunks, st = g % NSTAGE, ps = g / KSTAGE_CHUNKS, buf = ps & 1;
+                    if (g % KSTAGE_CHUNKS == 0 && ps >= 2 && !mbar_wait(acce0 + 8 * buf, ((ps >> 1) - 1) & 1)) { *abort_flag = 1; go = false; break; }
+                    if (!mbar_wait(full0 + 8 * st, (g / NSTAGE) & 1)) { *abort_flag = 1; go = false; break; }
+                    if (*abort_flag) { go = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t a0 = smem0 + st * STAGE_BYTES, b0 = a0 + A_CHUNK_BYTES;
+                    const uint32_t d0 = tmem + (uint32_t)buf * ACC_COLS;
 #pragma unroll
-                for (int h = 0; h < KCH / 16; ++h) {
+                    for (int h = 0; h < KCH / 16; ++h) {
 #pragma unroll
-                    for (int p = 1; p <= SL; ++p) {
-                        const uint32_t acc = (c % KSTAGE_CHUNKS == 0 && h == 0 && p == 1) ? 0u : 1u;
-                        mma_bf16(d0 + (uint32_t)(p - 1) * TN, make_desc(a0 + (p - 1) * A_SLICE_BYTES + h * 256),
-                                 make_desc(b0 + h * 256), idesc_bf16((uint32_t)(n_q(p) * TN)), acc);
+                        for (int p = 1; p <= SL; ++p) {
+                            const uint32_t acc = (g % KSTAGE_CHUNKS == 0 && h == 0 && p == 1) ? 0u : 1u;
+                            mma_bf16(d0 + (uint32_t)(p - 1) * TN, make_desc(a0 + (p - 1) * A_SLICE_BYTES + h * 256),
+                                     make_desc(b0 + h * 256), idesc_bf16((uint32_t)(n_q(p) * TN)), acc);
+                        }
                     }
+                    mma_commit(empty0 + 8 * st);
+                    if (g % KSTAGE_CHUNKS == KSTAGE_CHUNKS - 1) mma_commit(accf0 + 8 * buf);
+                    mma_chunks = g + 1;
                 }
-                mma_commit(empty0 + 8 * st);
-                if (c % KSTAGE_CHUNKS == KSTAGE_CHUNKS - 1) mma_commit(accf0 + 8 * buf);
-                mma_chunks = c + 1;
             }
         }
     } else {
@@ -423,13 +436,19 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const GemmArgs G) {
         // running sums of the two diagonal groups, folded per stage:
         //   hi += D2 2^21 + D3 2^14 + D4 2^7 + D5,  lo += D6 2^21 + D7 2^14 + D8 2^7 + D9
         // (|D_t| < 2^24 per stage, so each stage adds < 2^45.1 and 2^51 bounds any K here)
+        int ps = 0;              // stages drained
+        bool ok = true;
+        for (int q = blockIdx.x; q < ntiles && ok; q += gridDim.x) {
+        Tile T;
+        if (!tile_of(G, q, ctiles, T)) continue;
+        const int ct = T.ct, rt = T.rt, node = T.node, e_act = T.e_act, aitem = T.aitem;
+        const int pe = ps + T.nseg * KC / KSTAGE_CHUNKS;
         long long acc[2][16];
 #pragma unroll
         for (int g = 0; g < 2; ++g)
 #pragma unroll
             for (int j = 0; j < 16; ++j) acc[g][j] = 0;
-        bool ok = true;
-        for (int ps = 0; ps < nstages; ++ps) {
+        for (; ps < pe; ++ps) {
             const int buf = ps & 1;
             if (!mbar_wait(accf0 + 8 * buf, (ps >> 1) & 1)) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;");
@@ -458,34 +477,57 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const GemmArgs G) {
             const int rp = rt * TM + quarter * 32 + lane;       // real row of this thread
             const int r = rp >> 1, part = rp & 1;
             const int ebias = G.rexp[(size_t)aitem * 2 * n_pad + rp];
-            if (r < n) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int col = ct * TN + half * 16 + j;
-                    const int k = col / m, g = col % m;
-                    if (k >= G.n_act || (e_act >= 0 && k != e_act) || col < G.col_lo || col >= G.col_hi) continue;
-                    const int fe = G.fexp[col];
-                    const int e = G.act[k];
-                    const ResJob& J = G.jobs[e];
-                    if (g >= J.ms + J.md) continue;
-                    double P = 0.0;
-                    if (fe > 0 && ebias > 0) {
-                        const long long hi = acc[0][j], lo = acc[1][j];
-                        // scale 2^(e_row + f_col) with e = ebias - 1022, f = fe - 1022
-                        const int sc = (ebias - 1022) + (fe - 1022);
-                        P = fma((double)lo, pow2(sc - 63), (double)hi * pow2(sc - 35));
-                    }
-                    double* R = reinterpret_cast<double*>(G.R + e * G.sC + ((size_t)node * n + r) * m + g) + part;
-                    if (G.mode == MODE_M) {
-                        double b = 0.0;
-                        if (node == 0 && g < J.ms) { const double2 bv = J.rhs_s[(size_t)r * J.ms + g]; b = part ? bv.y : bv.x; }
-                        if (node == N - 1 && g >= J.ms) { const double2 bv = J.rhs_d[(size_t)r * J.md + (g - J.ms)]; b = part ? bv.y : bv.x; }
-                        *R = fma(-J.E, P, b);
-                    } else {
-                        *R += P;
-                    }
+            // lane j (and j + 16) looks column j up once: energy, place in R, exponent, right-hand
+            // side (end nodes of the M product); the columns' owners are broadcast below.  (Each
+            // thread looking up all 16, three dependent loads each, took half of a tile's time.)
+            const int col = ct * TN + half * 16 + (lane & 15), k = col / m, g = col % m;
+            long long off = -1, rhs = 0;
+            int fe = 0, ldb = 0;
+            double Ej = 0.0;
+            if (k < G.n_act && (e_act < 0 || k == e_act) && col >= G.col_lo && col < G.col_hi) {
+                const int e = G.act[k];
+                const ResJob& J = G.jobs[e];
+                if (g < J.ms + J.md) {
+                    off = e * G.sC + (long long)node * n * m + g;
+                    fe = G.fexp[col];
+                    Ej = J.E;
+                    if (G.mode == MODE_M && node == 0 && g < J.ms) { rhs = reinterpret_cast<long long>(J.rhs_s + g); ldb = J.ms; }
+                    if (G.mode == MODE_M && node == N - 1 && g >= J.ms) { rhs = reinterpret_cast<long long>(J.rhs_d + (g - J.ms)); ldb = J.md; }
                 }
             }
+            const bool row = r < n, add = G.mode != MODE_M;
+            double* R = reinterpret_cast<double*>(G.R) + 2 * (long long)r * m + part;
+            double old[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const long long o = __shfl_sync(0xffffffffu, off, j);
+                old[j] = add && row && o >= 0 ? R[2 * o] : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const long long o = __shfl_sync(0xffffffffu, off, j), bp = __shfl_sync(0xffffffffu, rhs, j);
+                const int f = __shfl_sync(0xffffffffu, fe, j), lb = __shfl_sync(0xffffffffu, ldb, j);
+                const double E = __shfl_sync(0xffffffffu, Ej, j);
+                if (!row || o < 0) continue;
+                double P = 0.0;
+                if (f > 0 && ebias > 0) {
+                    const long long hi = acc[0][j], lo = acc[1][j];
+                    // scale 2^(e_row + f_col) with e = ebias - 1022, f = fe - 1022
+                    const int sc = (ebias - 1022) + (f - 1022);
+                    P = fma((double)lo, pow2(sc - 63), (double)hi * pow2(sc - 35));
+                }
+                if (!add) {
+                    double b = 0.0;
+                    if (bp) {
+                        const double2 bv = reinterpret_cast<const double2*>(bp)[(size_t)r * lb];
+                        b = part ? bv.y : bv.x;
+                    }
+                    R[2 * o] = fma(-E, P, b);
+                } else {
+                    R[2 * o] = old[j] + P;
+                }
+            }
+        }
         }
     }
     // ---------------- teardown: every copy and MMA of this CTA must have landed
@@ -608,8 +650,11 @@ void gemm(const GemmArgs& G, int items, cudaStream_t st) {
     else if (G.col_lo > 0 || G.col_hi < G.nct * TN)                                // one system's columns
         tiles = std::min(G.nct, (std::min(G.col_hi, G.nct * TN) - 1) / TN - G.col_lo / TN + 1);
     if (tiles <= 0 || items <= 0) return;
-    dim3 grid(tiles, 2 * n_pad / TM, items);
-    k_oz_gemm<<<grid, THREADS, SMEM_BYTES, st>>>(G);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int ntiles = tiles * (2 * n_pad / TM) * items;
+    k_oz_gemm<<<std::min(ntiles, sms), THREADS, SMEM_BYTES, st>>>(G, tiles, ntiles);
 }
 
 void norms(const double2* R, long long sC, const ResJob* jobs, const int* act, int n_act, int n, int N, int m, cudaStream_t st) {
