@@ -181,6 +181,11 @@ struct pwqt_ctx {
     // grow-only workspaces of the sweep (kept across calls: no allocation in steady state)
     pwqt::DBuf ws_xy, ws_s, ws_norms, ws_jobs, ws_obs, ws_res, ws_mixed, ws_dens;
     pwqt::DBuf zero_nn;   // n x n zeros
+    // results of a host-buffer call on the device and, page-locked, on the host (grow-only, at
+    // most OUT_HOST_MAX bytes on the host)
+    pwqt::DBuf ws_out;
+    void* out_host = nullptr;
+    size_t out_host_bytes = 0;
     // optional CUDA-event timing of the dominant (block-sweep) kernels
     int profile = 0;
     double prof_ms = 0.0;
@@ -201,6 +206,7 @@ struct pwqt_ctx {
     // the two halves of a mixed-precision batch (lane 0 also serves undivided batches)
     pwqt::Lane lanes[2];
     ~pwqt_ctx() {
+        if (out_host) cudaFreeHost(out_host);
         for (auto& w : workers) w->destroy();
         for (auto& l : lanes) l.destroy();
     }

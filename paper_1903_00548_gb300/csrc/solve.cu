@@ -178,14 +178,35 @@ int solve_batch(pwqt_ctx* c, System& s, int nE, const double* E, int precision, 
             for (int e = 0; e < nE; ++e) PWQT_TRY(mixed_prepare(c, *sys_of[e], st));
         }
     }
-    size_t free_b = 0, total_b = 0;
-    PWQT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
-    size_t budget = c->opts.hbm_budget_bytes ? c->opts.hbm_budget_bytes : (size_t)(0.85 * (double)free_b);
     auto per_energy = [&](int e) {
         int m = ms[e] + md[e];
         if (precision != PWQT_FP64) return mixed_bytes_per_energy(n, N, std::max(m, 1)) + 64 * sizeof(double) * (m + 2);
         return sizeof(double2) * ((size_t)N * n * (n + m) + nn) + 64 * sizeof(double) * (m + 2);
     };
+    // the free memory is asked for (some 0.1 ms) only when the workspaces do not hold the whole
+    // call already
+    size_t budget = c->opts.hbm_budget_bytes;
+    if (!budget) {
+        size_t need = 0, xy = 0;
+        int mx = 1;
+        for (int e = 0; e < nE; ++e) {
+            need += per_energy(e);
+            xy += sizeof(double2) * (size_t)N * n * (n + ms[e] + md[e]);
+            mx = std::max(mx, ms[e] + md[e]);
+        }
+        bool held;
+        if (precision == PWQT_FP64) held = c->ws_xy.bytes >= xy && c->ws_s.bytes >= sizeof(double2) * nn * nE;
+        else {
+            const size_t half = mixed_bytes_per_energy(n, N, mx) * (size_t)(nE >= 16 ? nE - nE / 2 : nE) + 1024 * 4;
+            held = c->lanes[0].ws_mixed.bytes >= half && (nE < 16 || c->lanes[1].ws_mixed.bytes >= half);
+        }
+        budget = need;
+        if (!held) {
+            size_t free_b = 0, total_b = 0;
+            PWQT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
+            budget = (size_t)(0.85 * (double)free_b);
+        }
+    }
     SweepSys sys{n, N, c->M0.as<double2>(), c->M1.as<double2>(), s.HV0.as<double2>(), s.HV1.as<double2>()};
     // energies whose contacts failed the mode count get zero self-energies and no
     // injected modes (their status carries PWQT_ST_MODE_COUNT)
