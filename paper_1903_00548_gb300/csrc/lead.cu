@@ -727,6 +727,15 @@ int fill_leads(pwqt_ctx* c, const std::vector<double>& keys) {
             if (r != PWQT_OK) { rc[t] = r; errs[t] = local.err; break; }
         }
     };
+    // the first entry of a block size alone: it loads the solver's kernels of that size.  Left
+    // to several threads at once that has stood still (three times, each at the first use of
+    // n = 70 or 72 in a process with other contexts before; not since entries come first alone)
+    if (c->leads_n != c->n && miss.size() > 1) {
+        int r = compute_lead_shared(c, c, *c->workers[0], miss[0], res[0]);
+        if (r != PWQT_OK) return r;
+        next = 1;
+    }
+    c->leads_n = c->n;
     std::vector<std::thread> th;
     for (int t = 1; t < nthreads; ++t) th.emplace_back(work, t);
     work(0);
