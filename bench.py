@@ -430,7 +430,7 @@ def run_ours(args, world, rank, local):
     roof_sweep = {"bound": "tensor" if prec == pw.MIXED else "fp64",
                   "achieved": sweep_alg / (sweep_ms / 1e3) / 1e12 if sweep_ms else None,
                   "peak": tf32 if prec == pw.MIXED else f64_peak, "unit": "TFLOP/s",
-                  "kernel": "block sweep (k_cgemm_tc, k_mx_panel_blk, k_mx_panel_apply, k_mx_trsm_up)" if prec == pw.MIXED else "k_sweep_fp64",
+                  "kernel": "block sweep (k_cgemm_tc, k_mx_panel_reg, k_mx_panel_apply, k_mx_trsm_up)" if prec == pw.MIXED else "k_sweep_fp64",
                   "work": "(56/3) N n^3 real flop per energy (complex LU, X_i solve, Schur product)",
                   "peak_source": f"{src} bf16 x nominal {'tf32' if prec == pw.MIXED else 'f64'}/bf16", "traffic": None,
                   "ms_per_step": sweep_ms, "launches": sweep_n}
@@ -470,7 +470,7 @@ def run_ours(args, world, rank, local):
     roof = max(cand, key=lambda x: x[0])[1] if cand else roof_sweep
     if roof is not roof_sweep and sweep_ms > max(t for t, _ in cand):
         roof = dict(roof)
-        roof["note_step"] = (f"the block sweep (k_cgemm_tc, k_mx_panel_blk, k_mx_panel_apply, k_mx_trsm_up: "
+        roof["note_step"] = (f"the block sweep (k_cgemm_tc, k_mx_panel_reg, k_mx_panel_apply, k_mx_trsm_up: "
                              f"{sweep_ms:.0f} ms per step over its launches) is the largest phase; "
                              "its own object is roofline_sweep")
 

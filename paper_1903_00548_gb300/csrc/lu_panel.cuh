@@ -35,16 +35,12 @@ struct __align__(16) Cand {
     int row, zero;           // zero: u[0] is exactly zero
 };
 // what the panel warps share: candidates and their magnitudes, two columns in turn
-struct __align__(16) PanelMem { Cand c[2][8]; unsigned key[2][8]; float2 trash[NT]; };
+struct __align__(16) PanelMem { Cand c[2][4]; unsigned key[2][4]; float2 trash[128]; };
 
-// leading dimension of a factored panel (odd, so that its columns of one row sit in different
-// banks) and the shared memory of a block, in elements
-__host__ __device__ inline int ldp(int n) { return n | 1; }
-__host__ __device__ inline int block_elems(int n) { return ldp(n) * PB; }
 inline int blocks_of(int n) { return (n + PB - 1) / PB; }
 inline size_t smem_bytes(int n, int C) {
     const int bl = (blocks_of(n) + C - 1) / C;
-    return (size_t)(bl + 1) * block_elems(n) * sizeof(float2) + sizeof(PanelMem) + sizeof(int) * (n + 2 * PB);
+    return (size_t)(bl + 1) * n * PB * sizeof(float2) + sizeof(PanelMem) + sizeof(int) * (n + 2 * PB);
 }
 
 // u[k] of column `cl` of block V: the panel's 8 pivot rows through its unit lower triangle
@@ -57,7 +53,7 @@ __device__ __forceinline__ void pivot_rows(const float2* V, const float2* lp, in
 #pragma unroll
     for (int q = 0; q + 1 < PB; ++q)
 #pragma unroll
-        for (int k = q + 1; k < PB; ++k) u[k] = lu::fnma(u[k], lp[q * ldp(n) + p[k]], u[q]);
+        for (int k = q + 1; k < PB; ++k) u[k] = lu::fnma(u[k], lp[q * n + p[k]], u[q]);
 }
 
 // rows [r0, r1) of B neighbouring local blocks at V: V[r][.] -= l[r][.] u, rows used as pivots
@@ -73,13 +69,13 @@ __device__ __forceinline__ void update_rows(float2* V, const float2* lp, int n, 
         for (int q = 0; q < 4; ++q) {
             x[q] = min(r + 4 * q, n - 1);
 #pragma unroll
-            for (int b = 0; b < B; ++b) v[q][b] = V[b * block_elems(n) + x[q] * PB + cl];
+            for (int b = 0; b < B; ++b) v[q][b] = V[((size_t)b * n + x[q]) * PB + cl];
         }
 #pragma unroll
         for (int k = 0; k < PB; ++k)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float2 l = lp[k * ldp(n) + x[q]];
+                const float2 l = lp[k * n + x[q]];
 #pragma unroll
                 for (int b = 0; b < B; ++b) v[q][b] = lu::fnma(v[q][b], l, u[b][k]);
             }
@@ -87,7 +83,7 @@ __device__ __forceinline__ void update_rows(float2* V, const float2* lp, int n, 
         for (int q = 0; q < 4; ++q)
             if (r + 4 * q < r1 && step[x[q]] < 0)
 #pragma unroll
-                for (int b = 0; b < B; ++b) V[b * block_elems(n) + x[q] * PB + cl] = v[q][b];
+                for (int b = 0; b < B; ++b) V[((size_t)b * n + x[q]) * PB + cl] = v[q][b];
     }
 }
 
@@ -97,9 +93,9 @@ template <int B>
 __device__ __forceinline__ void update_blocks(float2* V, const float2* lp, float2* F, int n, const int* pv, const int* step, int p, int x,
                                               int C, int rank, int r0, int r1, int lane) {
     float2 u[B][PB];
-    float2* Q = V + (size_t)x * block_elems(n);
+    float2* Q = V + (size_t)x * n * PB;
 #pragma unroll
-    for (int b = 0; b < B; ++b) pivot_rows(Q + b * block_elems(n), lp, n, pv, lane & 7, u[b]);
+    for (int b = 0; b < B; ++b) pivot_rows(Q + (size_t)b * n * PB, lp, n, pv, lane & 7, u[b]);
     update_rows<B>(Q, lp, n, step, u, r0, r1, lane);
     if (r0 == 0 && lane < PB)
 #pragma unroll
@@ -112,7 +108,7 @@ __device__ __forceinline__ void update_blocks(float2* V, const float2* lp, float
 }
 
 // W warps (threads 0 .. 32 W - 1, RPL rows a lane): the panel V (n rows, wd columns) with
-// the rows marked in step already used, left as V[k ldp(n) + r]; its pivots to pv (a NaN counts
+// the rows marked in step already used, left as V[k n + r]; its pivots to pv (a NaN counts
 // as the largest).  Returns whether a pivot was exactly zero.
 template <int W, int RPL>
 __device__ __forceinline__ int factor_panel(float2* V, const int* step, int n, int wd, int* pv, PanelMem& pm) {
@@ -172,14 +168,7 @@ __device__ __forceinline__ int factor_panel(float2* V, const int* step, int n, i
             unsigned best = kk.x;
             if (kk.y > best) { best = kk.y; w = 1; }
             if (W > 2 && kk.z > best) { best = kk.z; w = 2; }
-            if (W > 3 && kk.w > best) { best = kk.w; w = 3; }
-            if (W > 4) {
-                const uint4 k2 = *reinterpret_cast<const uint4*>(pm.key[par] + 4);
-                if (k2.x > best) { best = k2.x; w = 4; }
-                if (k2.y > best) { best = k2.y; w = 5; }
-                if (k2.z > best) { best = k2.z; w = 6; }
-                if (k2.w > best) w = 7;
-            }
+            if (W > 3 && kk.w > best) w = 3;
         }
         const Cand& s = pm.c[par][w];
         float2 u[PB];
@@ -200,7 +189,7 @@ __device__ __forceinline__ int factor_panel(float2* V, const int* step, int n, i
             // no branch: rows that are done get a zero multiplier, those past n go to trash
             const bool on = !((done >> q) & 1u);
             float2 l = lu::mul(a[q][0], iv);
-            *(r < n ? V + k * ldp(n) + r : pm.trash + t) = on ? l : a[q][0];
+            *(r < n ? V + k * n + r : pm.trash + t) = on ? l : a[q][0];
             l = on ? l : make_float2(0.f, 0.f);
 #pragma unroll
             for (int c = 1; c < PB; ++c) a[q][c - 1] = lu::fnma(a[q][c], l, u[c]);
@@ -224,15 +213,15 @@ __global__ void __launch_bounds__(NT) k_lu_panel(Batch B, int n) {
     const int e = blockIdx.x / C, t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int nbk = (n + PB - 1) / PB, bl = (nbk + (int)C - 1) / (int)C, own = (nbk - (int)rank + (int)C - 1) / (int)C;
     float2* F = B.S + e * B.stride;
-    float2* V = lsm;                                // local block x: V + x block_elems(n)
-    float2* lbuf = lsm + (size_t)bl * block_elems(n);       // the panel in use (C > 1)
-    PanelMem& pm = *reinterpret_cast<PanelMem*>(lbuf + block_elems(n));
+    float2* V = lsm;                                // local block x: V + x n PB
+    float2* lbuf = lsm + (size_t)bl * n * PB;       // the panel in use (C > 1)
+    PanelMem& pm = *reinterpret_cast<PanelMem*>(lbuf + (size_t)n * PB);
     int* step = reinterpret_cast<int*>(&pm + 1);
     int* pv = step + n;                             // pivots of the panel this CTA factored
     int* cur = pv + PB;                             // pivots of the panel in use
     for (int q = t; q < own * n * PB; q += NT) {
         const int c = q % PB, x = (q / PB) % own, r = q / (PB * own), col = (x * (int)C + (int)rank) * PB + c;
-        V[(size_t)x * block_elems(n) + r * PB + c] = col < n ? F[(size_t)r * n + col] : make_float2(0.f, 0.f);
+        V[((size_t)x * n + r) * PB + c] = col < n ? F[(size_t)r * n + col] : make_float2(0.f, 0.f);
     }
     for (int r = t; r < n; r += NT) step[r] = -1;
     __syncthreads();
@@ -244,13 +233,13 @@ __global__ void __launch_bounds__(NT) k_lu_panel(Batch B, int n) {
         if (C > 1) lu::cl_sync();
         else __syncthreads();
         // the factored panel and its pivots
-        const float2* panel = V + (size_t)(p / (int)C) * block_elems(n);
+        const float2* panel = V + (size_t)(p / (int)C) * n * PB;
         const int* ppv = pv;
         if (C > 1) {
-            const float4* src = reinterpret_cast<const float4*>(lu::cl_map(V + (size_t)(p / (int)C) * block_elems(n), (uint32_t)owner));
+            const float4* src = reinterpret_cast<const float4*>(lu::cl_map(V + (size_t)(p / (int)C) * n * PB, (uint32_t)owner));
             ppv = lu::cl_map(pv, (uint32_t)owner);
             if ((int)rank != owner) {
-                for (int q = t; q < block_elems(n) / 2; q += NT) reinterpret_cast<float4*>(lbuf)[q] = src[q];
+                for (int q = t; q < n * PB / 2; q += NT) reinterpret_cast<float4*>(lbuf)[q] = src[q];
                 panel = lbuf;
             }
         }
@@ -265,7 +254,7 @@ __global__ void __launch_bounds__(NT) k_lu_panel(Batch B, int n) {
         const int xn = (p + 1) / (int)C;
         if (next) {
             // the next panel first, a share of its rows per warp
-            float2* Q = V + (size_t)xn * block_elems(n);
+            float2* Q = V + (size_t)xn * n * PB;
             const int share = ((n + 7) / 8 + 3) / 4 * 4;
             update_blocks<1>(V, panel, F, n, cur, step, p, xn, (int)C, (int)rank, warp * share, min(n, (warp + 1) * share), lane);
             __syncthreads();
@@ -285,7 +274,7 @@ __global__ void __launch_bounds__(NT) k_lu_panel(Batch B, int n) {
     // L, and U inside the panels' diagonal blocks
     for (int q = t; q < own * n * PB; q += NT) {
         const int c = q % PB, x = (q / PB) % own, r = q / (PB * own), k0 = (x * (int)C + (int)rank) * PB;
-        if (k0 + c < n && step[r] >= k0) F[(size_t)step[r] * n + k0 + c] = V[(size_t)x * block_elems(n) + c * ldp(n) + r];
+        if (k0 + c < n && step[r] >= k0) F[(size_t)step[r] * n + k0 + c] = V[((size_t)x * PB + c) * n + r];
     }
     if (rank == 0) {
         int* perm = B.perm + e * B.sperm;

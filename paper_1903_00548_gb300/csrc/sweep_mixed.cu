@@ -22,7 +22,6 @@
 #include <cstdint>
 
 #include "cgemm_tc.cuh"
-#include "lu_panel.cuh"
 #include "residual_oz.cuh"
 #include "sweep_c64.cuh"
 #include "sweep_mixed.cuh"
@@ -208,81 +207,136 @@ __global__ void __launch_bounds__(NT) k_mx_panel(MixSys S, int i, int k0, int wd
     }
 }
 
-// k_mx_panel for panels that fit shared memory so (up to about 830 rows): four blocks of 8 columns, each
-// factored in the registers of all 8 warps (lu_panel.cuh) and applied to the blocks right
-// of it.  Rows are not moved meanwhile; at the end the pivots are turned into the swaps that
-// k_mx_panel records, and rows are written where those put them.  A column costs about 500
-// cycles; with a thread owning two 32-column rows and the pivot rows exchanged through
-// shared memory it was 5500 (92 us a panel at 16 energies).
-template <int RPL>
-__global__ void __launch_bounds__(NT) k_mx_panel_blk(MixSys S, int i, int k0, int wd) {
-    extern __shared__ __align__(16) float2 P[];
-    const int e = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int n = S.n, rows = n - k0, be = lup::block_elems(rows), lp = lup::ldp(rows);
+// k_mx_panel for panels of at most 512 rows: the panel in registers (thread t holds panel
+// rows t and t + 256, all 32 columns), so the rank-1 updates touch no shared memory; per
+// column the pivot (max |re|+|im|, the lower row on ties, as k_mx_panel) is found by warp
+// shuffles and one pass over the warps' candidates, and rows j and p are exchanged and
+// the pivot row broadcast through shared memory.  Pivots, the factored panel and the list
+// of row moves are written as k_mx_panel writes them.
+constexpr int PR_NT = 256;
+__global__ void __launch_bounds__(PR_NT) k_mx_panel_reg(MixSys S, int i, int k0, int wd) {
+    __shared__ float2 prow_s[PW], jrow_s[PW];
+    __shared__ float bv[PR_NT / 32];
+    __shared__ int bi[PR_NT / 32], prow[PW], sel;
+    const int e = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int n = S.n, rows = n - k0;
     float2* F = S.F + e * S.sF + (size_t)i * n * n + (size_t)k0 * n + k0;   // panel origin, row stride n
     int* piv = S.piv + e * S.sP + (size_t)i * n;
-    float2* U = P + 4 * (size_t)be;                            // U right of a diagonal block, 32 x 32
-    lup::PanelMem& pm = *reinterpret_cast<lup::PanelMem*>(U + PW * PW);
-    int* step = reinterpret_cast<int*>(&pm + 1);
-    int* orig = step + rows;                                   // row at a position, after the swaps so far
-    int* pos = orig + rows;
-    int* prow = pos + rows;                                    // pivot row of a step
-    int* pv = prow + PW;
-    __shared__ int mvc;
-    for (int q = t; q < rows * PW; q += NT) {
-        const int r = q / PW, c = q % PW;
-        P[(c >> 3) * be + r * lup::PB + (c & 7)] = c < wd ? F[(size_t)r * n + c] : make_float2(0.f, 0.f);
+    float2 a[2][PW];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int r = t + q * PR_NT;
+#pragma unroll
+        for (int c = 0; c < PW; ++c) a[q][c] = (r < rows && c < wd) ? F[(size_t)r * n + c] : make_float2(0.f, 0.f);
     }
-    for (int r = t; r < rows; r += NT) { step[r] = -1; orig[r] = r; pos[r] = r; }
+    int st = 0;
+#pragma unroll
+    for (int j = 0; j < PW; ++j) {
+        if (j >= wd) break;
+        float best = -1.f;
+        int idx = j;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int r = t + q * PR_NT;
+            if (r >= j && r < rows) {
+                const float v = fabsf(a[q][j].x) + fabsf(a[q][j].y);
+                if (v > best) { best = v; idx = r; }
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_down_sync(0xffffffffu, best, o);
+            const int oi = __shfl_down_sync(0xffffffffu, idx, o);
+            if (ov > best || (ov == best && oi < idx)) { best = ov; idx = oi; }
+        }
+        if (lane == 0) { bv[warp] = best; bi[warp] = idx; }
+        __syncthreads();
+        if (t == 0) {
+            float b = bv[0];
+            int ii = bi[0];
+            for (int q = 1; q < PR_NT / 32; ++q)
+                if (bv[q] > b || (bv[q] == b && bi[q] < ii)) { b = bv[q]; ii = bi[q]; }
+            const int p = b < 0.f ? j : ii;   // no candidate rows: keep the diagonal
+            sel = p;
+            prow[j] = p;
+            piv[k0 + j] = k0 + p;
+        }
+        __syncthreads();
+        const int p = sel;
+        // the owners publish row p (the pivot row) and, if different, row j
+        if (t == p % PR_NT) {
+            const bool hi = p >= PR_NT;
+#pragma unroll
+            for (int c = 0; c < PW; ++c) prow_s[c] = hi ? a[1][c] : a[0][c];
+        }
+        if (p != j && t == j) {
+#pragma unroll
+            for (int c = 0; c < PW; ++c) jrow_s[c] = a[0][c];
+        }
+        __syncthreads();
+        if (p != j) {
+            if (t == j)
+#pragma unroll
+                for (int c = 0; c < PW; ++c) a[0][c] = prow_s[c];
+            if (t == p % PR_NT) {
+                if (p >= PR_NT) {
+#pragma unroll
+                    for (int c = 0; c < PW; ++c) a[1][c] = jrow_s[c];
+                } else {
+#pragma unroll
+                    for (int c = 0; c < PW; ++c) a[0][c] = jrow_s[c];
+                }
+            }
+        }
+        float2 pv = prow_s[j];
+        if (pv.x == 0.f && pv.y == 0.f) { st |= PWQT_ST_SINGULAR_PIVOT; pv = make_float2(1.f, 0.f); }
+        const float2 inv = fdiv(make_float2(1.f, 0.f), pv);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int r = t + q * PR_NT;
+            if (r > j && r < rows) {
+                const float2 x = a[q][j];
+                const float2 l = make_float2(x.x * inv.x - x.y * inv.y, x.x * inv.y + x.y * inv.x);
+                a[q][j] = l;
+#pragma unroll
+                for (int c = j + 1; c < PW; ++c) {
+                    const float2 u = prow_s[c];
+                    ffma(a[q][c], make_float2(-l.x, -l.y), u);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int r = t + q * PR_NT;
+        if (r < rows)
+#pragma unroll
+            for (int c = 0; c < PW; ++c)
+                if (c < wd) F[(size_t)r * n + c] = a[q][c];
+    }
+    // the swaps in order, as a map panel row -> original row; rows with a new origin (at
+    // most 2 wd) become the move list
+    __shared__ int orig[2 * PR_NT], mvc;
+    for (int r = t; r < rows; r += PR_NT) orig[r] = r;
     if (t == 0) mvc = 0;
     __syncthreads();
-    int bad = 0;
-    for (int b = 0; b * lup::PB < wd; ++b) {
-        const int wb = min(lup::PB, wd - b * lup::PB);
-        float2* V = P + (size_t)b * be;
-        bad |= lup::factor_panel<8, RPL>(V, step, rows, wb, pv, pm);
-        __syncthreads();
-        if (t < wb) {
-            step[pv[t]] = b * lup::PB + t;
-            prow[b * lup::PB + t] = pv[t];
+    if (t == 0)
+        for (int j = 0; j < wd; ++j) {
+            const int p = prow[j];
+            if (p != j) { const int x = orig[j]; orig[j] = orig[p]; orig[p] = x; }
         }
-        __syncthreads();
-        if (t == 0)                // this block's swaps, while the other warps update
-            for (int j = b * lup::PB; j < b * lup::PB + wb; ++j) {
-                const int r = prow[j], p = pos[r], o = orig[j];
-                piv[k0 + j] = k0 + p;
-                orig[j] = r; orig[p] = o;
-                pos[r] = j; pos[o] = p;
-            }
-        const int share = ((rows + 7) / 8 + 3) / 4 * 4, r0 = warp * share, r1 = min(rows, r0 + share);
-        for (int x = b + 1; x * lup::PB < wd; ++x) {          // a later block exists: this one is whole
-            float2 u[1][lup::PB];
-            lup::pivot_rows(P + (size_t)x * be, V, rows, prow + b * lup::PB, lane & 7, u[0]);
-            lup::update_rows<1>(P + (size_t)x * be, V, rows, step, u, r0, r1, lane);
-            if (warp == 1 && lane < lup::PB)
-#pragma unroll
-                for (int k = 0; k < lup::PB; ++k) U[(b * lup::PB + k) * PW + x * lup::PB + lane] = u[0][k];
-        }
-        __syncthreads();
-    }
+    __syncthreads();
     int* mv = S.mv + (size_t)e * MV_INTS;
-    for (int q = t; q < rows * PW; q += NT) {
-        const int y = q / PW, c = q % PW, r = orig[y];
-        if (c < wd) F[(size_t)y * n + c] = step[r] >= 0 && step[r] < (c & ~7) ? U[step[r] * PW + c] : P[(size_t)(c >> 3) * be + (c & 7) * lp + r];
-        if (c == 0 && r != y) {
+    for (int r = t; r < rows; r += PR_NT)
+        if (orig[r] != r) {
             const int k = atomicAdd(&mvc, 1);
-            mv[1 + k] = y;
-            mv[1 + 2 * PW + k] = r;
+            mv[1 + k] = r;
+            mv[1 + 2 * PW + k] = orig[r];
         }
-    }
     __syncthreads();
     if (t == 0) {
         mv[0] = mvc;
-        if (bad) atomicOr(S.jobs[e].status, PWQT_ST_SINGULAR_PIVOT);
+        if (st) atomicOr(S.jobs[e].status, st);
     }
-}
-size_t panel_blk_smem(int rows) {
-    return sizeof(float2) * (4 * (size_t)lup::block_elems(rows) + PW * PW) + sizeof(lup::PanelMem) + sizeof(int) * (3 * (size_t)rows + PW + lup::PB);
 }
 
 // The panel's row moves on the other columns of F_i and on XY_i (one column per thread,
@@ -955,9 +1009,6 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
     const int dyn_panel = smem_optin - (int)fa_panel.sharedSizeBytes;
     if (panel_smem > (size_t)dyn_panel) return fail(c, PWQT_ERR_INVALID_ARG, "panel exceeds shared memory");
     PWQT_CUDA(c, cudaFuncSetAttribute(k_mx_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_panel));
-    const int dyn_blk = smem_optin - 16;      // k_mx_panel_blk's one static word, rounded up
-    PWQT_CUDA(c, cudaFuncSetAttribute(k_mx_panel_blk<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_blk));
-    PWQT_CUDA(c, cudaFuncSetAttribute(k_mx_panel_blk<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_blk));
     auto gemm = [&](const float2* A, long long sA, int lda, const float2* B1, long long sB1, int ldb1, const float2* B2, long long sB2,
                     int ldb2, float2* C1, long long sC1, int ldc1, float2* C2, long long sC2, int ldc2, int split, int M, int Nc, int K) {
         CGemmArgs g{A, sA, lda, B1, sB1, ldb1, B2, sB2, ldb2, C1, sC1, ldc1, C2, sC2, ldc2, split};
@@ -975,9 +1026,7 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
         }
         for (int k0 = 0; k0 < n; k0 += PW) {
             const int wd = std::min(PW, n - k0);
-            const int rows = n - k0;
-            if (rows <= 512) k_mx_panel_blk<2><<<nb, NT, panel_blk_smem(rows), st>>>(S, i, k0, wd);
-            else if (panel_blk_smem(rows) <= (size_t)dyn_blk) k_mx_panel_blk<4><<<nb, NT, panel_blk_smem(rows), st>>>(S, i, k0, wd);
+            if (n - k0 <= 2 * PR_NT) k_mx_panel_reg<<<nb, PR_NT, 0, st>>>(S, i, k0, wd);
             else k_mx_panel<<<nb, NT, sizeof(float2) * (size_t)((n - k0) | 1) * PW, st>>>(S, i, k0, wd);
             k_mx_panel_apply<<<dim3((n - wd + w + APT - 1) / APT, nb), APT, 0, st>>>(S, i, k0, wd);
             c->launches += 2;
