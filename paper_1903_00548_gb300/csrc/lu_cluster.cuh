@@ -217,16 +217,17 @@ __global__ void __launch_bounds__(256) k_lu(Where where, int n) {
 #pragma unroll
         for (int x = 0; x < 4; ++x)
             if (j + 1 + t + x * NT < n) pv[x] = prow[j + 1 + t + x * NT];
-        // multipliers, a thread per part of a row's: l = a inv
-        for (int q = t >> 1; q < na; q += NT >> 1) {
-            const int r = ord[q];
-            if (mine && r == lr) continue;
-            T2* a = rows + (size_t)r * ldr + j;
-            const T2 v = *a;
-            const T l = (t & 1) ? fma(v.x, inv.y, v.y * inv.x) : fma(v.x, inv.x, -(v.y * inv.y));
-            reinterpret_cast<T*>(lm + r)[t & 1] = l;
-            __syncwarp(__activemask());
-            reinterpret_cast<T*>(a)[t & 1] = l;
+        // multipliers l = a inv, lanes 2q and 2q + 1 the real and imaginary part of one row's: a
+        // lane reads and writes its own part only and has the other by shuffle
+        for (int q0 = warp * 16; q0 < na; q0 += NT >> 1) {
+            const int q = q0 + (lane >> 1), part = lane & 1, r = ord[min(q, na - 1)];
+            T* a = reinterpret_cast<T*>(rows + (size_t)r * ldr + j) + part;
+            const T v = q < na ? *a : T(0), o = __shfl_xor_sync(0xffffffffu, v, 1);
+            const T l = part ? fma(o, inv.y, v * inv.x) : fma(v, inv.x, -(o * inv.y));
+            if (q < na && !(mine && r == lr)) {
+                reinterpret_cast<T*>(lm + r)[part] = l;
+                *a = l;
+            }
         }
 #pragma unroll
         for (int x = 0; x < 4; ++x)
