@@ -22,6 +22,7 @@
 #include <cmath>
 #include <thread>
 
+#include "first_use.h"
 #include "pwqt_internal.cuh"
 
 namespace pwqt {
@@ -704,6 +705,13 @@ int fill_leads(pwqt_ctx* c, const std::vector<double>& keys) {
     for (double k : keys)
         if (!c->cache.count(k) && std::find(miss.begin(), miss.end(), k) == miss.end()) miss.push_back(k);
     if (miss.empty()) return PWQT_OK;
+    // The process' first entry of a block size on a device alone, whatever the contexts and
+    // their threads.  With several threads at it a process has stood still three times (n = 70
+    // and 72, other contexts alive, the GPU answering); not since the first entry is alone.
+    // The cause is not known: the solver's kernels of a size are loaded then, beside the
+    // allocations and frees of the other threads' entries.
+    static FirstUse first_use;
+    FirstUse::Pass pass(first_use, c->dev, c->n);
     int nthreads = (int)std::min<size_t>(miss.size(), (size_t)std::max(1, c->lead_threads));
     while ((int)c->workers.size() < nthreads) {
         c->workers.emplace_back(new LeadWorker());
@@ -727,15 +735,11 @@ int fill_leads(pwqt_ctx* c, const std::vector<double>& keys) {
             if (r != PWQT_OK) { rc[t] = r; errs[t] = local.err; break; }
         }
     };
-    // the first entry of a block size alone: it loads the solver's kernels of that size.  Left
-    // to several threads at once that has stood still (three times, each at the first use of
-    // n = 70 or 72 in a process with other contexts before; not since entries come first alone)
-    if (c->leads_n != c->n && miss.size() > 1) {
-        int r = compute_lead_shared(c, c, *c->workers[0], miss[0], res[0]);
-        if (r != PWQT_OK) return r;
+    if (pass.first()) {
+        PWQT_TRY(compute_lead_shared(c, c, *c->workers[0], miss[0], res[0]));
         next = 1;
+        pass.known();
     }
-    c->leads_n = c->n;
     std::vector<std::thread> th;
     for (int t = 1; t < nthreads; ++t) th.emplace_back(work, t);
     work(0);

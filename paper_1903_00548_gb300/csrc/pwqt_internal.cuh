@@ -202,7 +202,6 @@ struct pwqt_ctx {
     cudaEvent_t ev2 = nullptr, ev3 = nullptr;
     // host threads that fill the contact cache concurrently
     int lead_threads = 8;
-    int leads_n = 0;                        // block size of the last contact entry
     std::vector<std::unique_ptr<pwqt::LeadWorker>> workers;
     // the two halves of a mixed-precision batch (lane 0 also serves undivided batches)
     pwqt::Lane lanes[2];
