@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/pwqt.h"
+#include "mixed_sizes.h"
 
 namespace pwqt {
 
@@ -146,6 +147,13 @@ struct Lane {
     long long prof_corr_launches = 0;
     int init(int dev);      // stream and events on first use
     void destroy();
+    MixedSizes sizes() const {      // of the buffers kept
+        MixedSizes s;
+        s.ws = ws_mixed.bytes;
+        s.sig_tab = oz_sig_tab.bytes; s.sig = oz_sig.bytes; s.sig_rexp = oz_sig_rexp.bytes;
+        s.B = oz_B.bytes; s.fexp = oz_fexp.bytes; s.act = oz_act.bytes;
+        return s;
+    }
 };
 }  // namespace pwqt
 

@@ -51,18 +51,11 @@ namespace pwqt {
 namespace oz {
 
 namespace {
-constexpr int SL = 7;                    // slices per operand
+// slices, tiles and chunks: mixed_sizes.h
 constexpr int TMAX = 9;                  // largest slice-index sum kept (p + q <= 9)
 constexpr int NDIAG = TMAX - 1;          // accumulators D_2 .. D_9
-constexpr int TM = 128;                  // real rows per tile
-constexpr int TN = 32;                   // columns per tile
-constexpr int KCH = 32;                  // real K per chunk (one bulk copy per operand)
 constexpr int KSTAGE_CHUNKS = 4;         // chunks per exact accumulation stage (128 real K)
 constexpr int NSTAGE = 3;                // shared-memory ring depth
-constexpr uint32_t A_SLICE_BYTES = TM * KCH * 2;          // 8 KB
-constexpr uint32_t B_SLICE_BYTES = TN * KCH * 2;          // 2 KB
-constexpr uint32_t A_CHUNK_BYTES = SL * A_SLICE_BYTES;    // 56 KB
-constexpr uint32_t B_CHUNK_BYTES = SL * B_SLICE_BYTES;    // 14 KB
 constexpr uint32_t B_STAGE_BYTES = B_CHUNK_BYTES + B_SLICE_BYTES;   // + the zero slice
 constexpr uint32_t STAGE_BYTES = A_CHUNK_BYTES + B_STAGE_BYTES;     // 72 KB
 constexpr uint32_t SMEM_BYTES = NSTAGE * STAGE_BYTES + 128;
@@ -614,20 +607,6 @@ int error_flag(bool reset, cudaStream_t st) {
     }
     return v;
 }
-
-int padded(int n) { return (n + 63) / 64 * 64; }
-
-size_t panel_bytes(int n, int items, int nseg) {
-    const int n_pad = padded(n);
-    return (size_t)items * (2 * n_pad / TM) * nseg * (2 * n_pad / KCH) * A_CHUNK_BYTES;
-}
-size_t panel_item_bytes(int n, int nseg) { return panel_bytes(n, 1, nseg); }
-size_t rexp_bytes(int n, int items) { return sizeof(int) * (size_t)items * 2 * padded(n); }
-size_t b_bytes(int n, int N, int ncols) {
-    const int n_pad = padded(n), nct = (ncols + TN - 1) / TN;
-    return (size_t)N * nct * (2 * n_pad / KCH) * B_CHUNK_BYTES;
-}
-int col_tiles(int ncols) { return (ncols + TN - 1) / TN; }
 
 void build_panel(const PanelSrc& P, int items, int* rexp, __nv_bfloat16* tiles, cudaStream_t st) {
     const int n_pad = padded(P.n);

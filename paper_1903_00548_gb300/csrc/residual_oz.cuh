@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "mixed_sizes.h"
 #include "sweep_mixed.cuh"
 
 namespace pwqt {
@@ -46,13 +47,6 @@ struct GemmArgs {
     int sigma_side;             // MODE_SIGMA: 0 source (node 0), 1 drain (node N-1); item = active energy
     int col_lo, col_hi;         // MODE_M / MODE_HV: the columns this launch writes (one system's energies)
 };
-
-int padded(int n);                                  // n rounded up to a multiple of 64
-int col_tiles(int ncols);
-size_t panel_bytes(int n, int items, int nseg);
-size_t panel_item_bytes(int n, int nseg);
-size_t rexp_bytes(int n, int items);
-size_t b_bytes(int n, int N, int ncols);
 
 int gemm_init();
 int error_flag(bool reset, cudaStream_t st);

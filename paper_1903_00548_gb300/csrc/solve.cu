@@ -184,21 +184,23 @@ int solve_batch(pwqt_ctx* c, System& s, int nE, const double* E, int precision, 
         return sizeof(double2) * ((size_t)N * n * (n + m) + nn) + 64 * sizeof(double) * (m + 2);
     };
     // the free memory is asked for (some 0.1 ms) only when the workspaces do not hold the whole
-    // call already
+    // call as one batch already, every buffer that grows with it among them
     size_t budget = c->opts.hbm_budget_bytes;
     if (!budget) {
         size_t need = 0, xy = 0;
-        int mx = 1;
+        std::vector<int> cols(nE);
         for (int e = 0; e < nE; ++e) {
+            cols[e] = ms[e] + md[e];
             need += per_energy(e);
-            xy += sizeof(double2) * (size_t)N * n * (n + ms[e] + md[e]);
-            mx = std::max(mx, ms[e] + md[e]);
+            xy += sizeof(double2) * (size_t)N * n * (n + cols[e]);
         }
-        bool held;
-        if (precision == PWQT_FP64) held = c->ws_xy.bytes >= xy && c->ws_s.bytes >= sizeof(double2) * nn * nE;
-        else {
-            const size_t half = mixed_bytes_per_energy(n, N, mx) * (size_t)(nE >= 16 ? nE - nE / 2 : nE) + 1024 * 4;
-            held = c->lanes[0].ws_mixed.bytes >= half && (nE < 16 || c->lanes[1].ws_mixed.bytes >= half);
+        bool held = c->opts.batch <= 0 || c->opts.batch >= nE;
+        if (precision == PWQT_FP64) {
+            held = held && c->ws_xy.bytes >= xy && c->ws_s.bytes >= sizeof(double2) * nn * nE;
+        } else {
+            MixedSizes kept[2];
+            for (int q = 0; q < 2; ++q) kept[q] = c->lanes[q].sizes();
+            held = held && lanes_hold(kept, n, N, nE, cols.data(), c->residual_kind == PWQT_RESIDUAL_SLICED);
         }
         budget = need;
         if (!held) {
@@ -334,13 +336,13 @@ int solve_batch(pwqt_ctx* c, System& s, int nE, const double* E, int precision, 
             PWQT_TRY(group(e0, nb, nullptr, st, obs_a));
         } else {
             PWQT_TRY(c->lanes[0].init(c->dev) == PWQT_OK ? PWQT_OK : fail(c, PWQT_ERR_CUDA, "lane stream"));
-            if (nb >= 16) {
+            split = lane_split(nb);
+            if (split < nb) {
                 // two halves on two lanes (streams, host threads): the GPU runs one half's
                 // residual and correction launches beside the other half's latency-bound sweep
                 // kernels.  While profiling, the halves run one after the other, so that each
                 // kernel's event time is its own and not the other lane's work on shared SMs.
                 PWQT_TRY(c->lanes[1].init(c->dev) == PWQT_OK ? PWQT_OK : fail(c, PWQT_ERR_CUDA, "lane stream"));
-                split = nb / 2;
                 PWQT_CUDA(c, cudaStreamSynchronize(st));   // work the halves depend on (zero block)
                 int rc_b = PWQT_OK;
                 auto run_b = [&] {

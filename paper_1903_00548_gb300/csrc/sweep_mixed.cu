@@ -30,9 +30,7 @@ namespace pwqt {
 
 namespace {
 
-constexpr int PW = 32;      // panel width
 constexpr int NT = 256;
-constexpr int MV_INTS = 4 * PW + 4;   // per energy: count, then 2 PW destination and 2 PW source rows
 constexpr int APT = 128;              // threads of the column-parallel panel kernels
 
 struct MixSys {
@@ -900,15 +898,6 @@ int corr_error_flag(bool reset, cudaStream_t st) {
 }
 }  // namespace
 
-size_t mixed_bytes_per_energy(int n, int N, int m) {
-    // F + XY + L_i (complex64) + pivots + FP64 solution and residual
-    const size_t w = (size_t)n + m + (m & 1);
-    return sizeof(float2) * ((size_t)N * n * n + (size_t)N * n * w + (size_t)N * n * n) + sizeof(int) * ((size_t)N * n + MV_INTS) + 256 +
-           3 * sizeof(double2) * (size_t)N * n * m +     // FP64 solution, residual, float-float copy
-           2 * oz::panel_item_bytes(n, 1) +               // self-energy slice panels
-           oz::b_bytes(n, N, m + 32);                     // solution slices (a column tile of slack)
-}
-
 int mixed_prepare(pwqt_ctx* c, System& s, cudaStream_t st) {
     if (c->residual_kind != PWQT_RESIDUAL_SLICED) return PWQT_OK;
     const int n = c->n, N = s.N;
@@ -963,8 +952,9 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
     S.sXY = (long long)N * n * w;
     S.sL = (long long)N * n * n;
     S.sC = (long long)N * n * m;
-    const size_t bytes = mixed_bytes_per_energy(n, N, m) * nb + 1024 * 4;
-    PWQT_TRY(ensure(c, L.ws_mixed, bytes));
+    const bool sliced = c->residual_kind == PWQT_RESIDUAL_SLICED;
+    const MixedSizes need = mixed_sizes(n, N, nb, m, sliced);
+    PWQT_TRY(ensure(c, L.ws_mixed, need.ws));
     char* base = L.ws_mixed.as<char>();
     auto take = [&](size_t b) { char* p = base; base += (b + 255) / 256 * 256; return p; };
     S.F = (float2*)take(sizeof(float2) * S.sF * nb);
@@ -1117,19 +1107,18 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
     // ---------------- the FP64-accurate residual on the tensor cores: self-energy panels
     // of this batch (slice tiles of Sigma_s, Sigma_d per energy), then per evaluation the
     // solution slices of the energies still refining and four slice-product launches
-    const bool sliced = c->residual_kind == PWQT_RESIDUAL_SLICED;
     oz::GemmArgs OG{};
     if (sliced) {
         if (oz::gemm_init() != 0) return fail(c, PWQT_ERR_CUDA, "slice-product GEMM set-up failed");
         if (!c->ozM.p || !s.ozH.p) return fail(c, PWQT_ERR_STATE, "slice panels missing (mixed_prepare)");
         std::vector<const double2*> tab(2 * nb);
         for (int b = 0; b < nb; ++b) { tab[2 * b] = jobs[b].sig_s; tab[2 * b + 1] = jobs[b].sig_d; }
-        PWQT_TRY(ensure(c, L.oz_sig_tab, sizeof(void*) * 2 * nb));
-        PWQT_TRY(ensure(c, L.oz_sig, oz::panel_bytes(n, 2 * nb, 1)));
-        PWQT_TRY(ensure(c, L.oz_sig_rexp, oz::rexp_bytes(n, 2 * nb)));
-        PWQT_TRY(ensure(c, L.oz_B, oz::b_bytes(n, N, nb * m)));
-        PWQT_TRY(ensure(c, L.oz_fexp, sizeof(int) * (size_t)oz::col_tiles(nb * m) * 32));
-        PWQT_TRY(ensure(c, L.oz_act, sizeof(int) * nb));
+        PWQT_TRY(ensure(c, L.oz_sig_tab, need.sig_tab));
+        PWQT_TRY(ensure(c, L.oz_sig, need.sig));
+        PWQT_TRY(ensure(c, L.oz_sig_rexp, need.sig_rexp));
+        PWQT_TRY(ensure(c, L.oz_B, need.B));
+        PWQT_TRY(ensure(c, L.oz_fexp, need.fexp));
+        PWQT_TRY(ensure(c, L.oz_act, need.act));
         PWQT_CUDA(c, cudaMemcpyAsync(L.oz_sig_tab.p, tab.data(), sizeof(void*) * 2 * nb, cudaMemcpyHostToDevice, st));
         oz::PanelSrc P{};
         P.n = n; P.nseg = 1;

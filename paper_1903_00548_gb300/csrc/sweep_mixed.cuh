@@ -2,6 +2,7 @@
 #pragma once
 #include <vector>
 
+#include "mixed_sizes.h"
 #include "pwqt_internal.cuh"
 #include "sweep_common.cuh"
 
@@ -43,7 +44,6 @@ void split_ff(const double2* in, float4* out, size_t count, cudaStream_t st);
 void launch_residual_ff(const ResidualFF& R, const ResJob* jobs, int nb, int m_max, const int* active, cudaStream_t st);
 void launch_residual_finish(const ResJob* jobs, int nb, cudaStream_t st, const int* active = nullptr);
 
-size_t mixed_bytes_per_energy(int n, int N, int m);
 // slice panels of the tensor-core residual for the basis and system (once; kept)
 int mixed_prepare(pwqt_ctx* c, System& s, cudaStream_t st);
 // sys_of[b]: the system of energy b of the batch (all with the same node count), or
