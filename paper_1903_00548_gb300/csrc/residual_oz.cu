@@ -443,7 +443,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const GemmArgs G, int ct
             for (int j = 0; j < 16; ++j) acc[g][j] = 0;
         for (; ps < pe; ++ps) {
             const int buf = ps & 1;
-            if (!mbar_wait(accf0 + 8 * buf, (ps >> 1) & 1)) { ok = false; break; }
+            // the warp gives up together: its reads of tensor memory and its broadcasts below take
+            // every lane
+            if (!__all_sync(0xffffffffu, mbar_wait(accf0 + 8 * buf, (ps >> 1) & 1))) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
