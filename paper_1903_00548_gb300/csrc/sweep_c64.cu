@@ -11,6 +11,12 @@
 // to stage, split and drain for a product that the FP32 pipes finish in 2, and the products
 // here round to nearest where the tensor cores' accumulation truncates.  D_i, U_i and L_i
 // are formed in FP64 (E M - HV) and rounded once.
+//
+// Sums of products are made 16 terms at a time and the partial sums added: a running sum over
+// all n terms left residuals of 1.3e-5 and 1.8e-5 at n = 128 and 320 (geometric mean of 8
+// energies, complex64 alone), above the tensor-core form's 9.3e-6, where this leaves 6.4e-6 and
+// 7.0e-6; the time is the same (n = 128, 200 nodes, 32 energies 134 -> 129 ms, n = 256 235 ->
+// 226, the tile kernel held to two CTAs an SM).
 #include <algorithm>
 
 #include "lu_panel.cuh"
@@ -57,7 +63,7 @@ __global__ void __launch_bounds__(256) k_c64_couplings(C64Sweep S) {
 // T x T tiles, T = 16 R, 256 threads with R x R outputs: S into F_i (column tiles first),
 // then the y columns (the source's; at the last node the drain's too)
 template <int R>
-__global__ void __launch_bounds__(256) k_c64_node(C64Sweep S, int i) {
+__global__ void __launch_bounds__(256, 2) k_c64_node(C64Sweep S, int i) {
     constexpr int T = 16 * R;
     __shared__ float2 As[T][17], Bs[16][T + 1];
     const int e = blockIdx.z;
@@ -95,6 +101,7 @@ __global__ void __launch_bounds__(256) k_c64_node(C64Sweep S, int i) {
             }
             __syncthreads();
             if (k0 + 16 < n) fetch(k0 + 16);
+            float2 part[R][R] = {};
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
                 float2 b[R];
@@ -104,9 +111,16 @@ __global__ void __launch_bounds__(256) k_c64_node(C64Sweep S, int i) {
                 for (int x = 0; x < R; ++x) {
                     const float2 a = As[ty + 16 * x][k];
 #pragma unroll
-                    for (int v = 0; v < R; ++v) fma2(acc[x][v], a, b[v]);
+                    for (int v = 0; v < R; ++v) fma2(part[x][v], a, b[v]);
                 }
             }
+#pragma unroll
+            for (int x = 0; x < R; ++x)
+#pragma unroll
+                for (int v = 0; v < R; ++v) {
+                    acc[x][v].x += part[x][v].x;
+                    acc[x][v].y += part[x][v].y;
+                }
         }
     }
     const double2* H = hv0(S, J, i);
@@ -162,12 +176,13 @@ template <int K> __device__ __forceinline__ void wait_groups() { asm volatile("c
 
 // rows r .. r+3 (those below `re`) of column c: X -= panel rows (P + (r - ra) SPL) x solved block xb
 __device__ __forceinline__ void solve_rows(float2* X, int CB, const float2* P, const float2* xb, int r, int re) {
-    float2 v[4];
+    float2 v[4], s[4];
     const float4* f[4];
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
         const int rr = min(x, re - 1 - r);
         v[x] = X[rr * CB];
+        s[x] = make_float2(0.f, 0.f);
         f[x] = reinterpret_cast<const float4*>(P + rr * SPL);
     }
 #pragma unroll
@@ -176,13 +191,13 @@ __device__ __forceinline__ void solve_rows(float2* X, int CB, const float2* P, c
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const float4 l = f[x][k];
-            v[x] = lu::fnma(v[x], make_float2(l.x, l.y), b0);
-            v[x] = lu::fnma(v[x], make_float2(l.z, l.w), b1);
+            fma2(s[x], make_float2(l.x, l.y), b0);
+            fma2(s[x], make_float2(l.z, l.w), b1);
         }
     }
 #pragma unroll
     for (int x = 0; x < 4; ++x)
-        if (r + x < re) X[x * CB] = v[x];
+        if (r + x < re) X[x * CB] = make_float2(v[x].x - s[x].x, v[x].y - s[x].y);
 }
 
 // 16 x 16 diagonal systems of up to two columns, a lane (hl) per row: D is the lane's row of
@@ -363,6 +378,7 @@ __global__ void __launch_bounds__(256) k_c64_back(C64Sweep S, int CB) {
                 const int r = q / cb * 4;
                 const float2* xb = cur + k * SP * CB + q % cb;
                 const float4* f[4];
+                float2 s[4] = {};
 #pragma unroll
                 for (int x = 0; x < 4; ++x) f[x] = reinterpret_cast<const float4*>(P + min(r + x, n - 1) * SPL);
 #pragma unroll
@@ -371,9 +387,14 @@ __global__ void __launch_bounds__(256) k_c64_back(C64Sweep S, int CB) {
 #pragma unroll
                     for (int x = 0; x < 4; ++x) {
                         const float4 l = f[x][z];
-                        v[b][x] = lu::fnma(v[b][x], make_float2(l.x, l.y), b0);
-                        v[b][x] = lu::fnma(v[b][x], make_float2(l.z, l.w), b1);
+                        fma2(s[x], make_float2(l.x, l.y), b0);
+                        fma2(s[x], make_float2(l.z, l.w), b1);
                     }
+                }
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    v[b][x].x -= s[x].x;
+                    v[b][x].y -= s[x].y;
                 }
             }
         }
