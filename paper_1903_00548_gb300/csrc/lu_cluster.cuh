@@ -1,9 +1,10 @@
-// LU factorisation of one n x n complex block per energy by a thread-block cluster.
+// LU factorisation of one n x n complex128 block per energy by a thread-block cluster (the
+// FP64 sweep's; the arithmetic helpers also serve the complex64 panels of lu_panel.cuh).
 //
 // The block's rows are dealt out over the cluster's C CTAs (row r to CTA r % C) and stay
 // in shared memory for the whole factorisation; nothing is exchanged but the pivot: per
-// column every CTA proposes its best row (max |re| + |im|), the winner's row is read through distributed shared memory, and each CTA updates its own
-// rows.  Rows are not moved: a row that has served as pivot is left alone, and at the end
+// column every CTA proposes its best row (max |re| + |im|), the winner's row is read through
+// distributed shared memory, and each CTA updates its own rows.  Rows are not moved: a row that has served as pivot is left alone, and at the end
 // row j of the factors is written from where the j-th pivot sat, with perm[j] its index
 // (the factors are those of P A, (P x)_j = x[perm[j]]; unit lower triangle).
 //
@@ -71,10 +72,6 @@ __device__ __forceinline__ unsigned long long mag_key(double v) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     return b <= 0x7ff0000000000000ull ? b + 2ull : 1ull;
 }
-__device__ __forceinline__ unsigned mag_key(float v) {
-    const unsigned b = __float_as_uint(v);
-    return b <= 0x7f800000u ? b + 2u : 1u;
-}
 // warp-wide: the first lane with the largest key
 __device__ __forceinline__ int warp_best(unsigned long long key) {
     const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
@@ -87,23 +84,19 @@ __device__ __forceinline__ int warp_best(unsigned key) {
     return __ffs(__ballot_sync(0xffffffffu, key == m)) - 1;
 }
 
-template <class T2> struct Key;
-template <> struct Key<double2> { using t = unsigned long long; };
-template <> struct Key<float2> { using t = unsigned; };
-
 // a CTA's proposal for one column: two 16-byte words
-template <class T2> struct __align__(16) Slot {
-    typename Key<T2>::t key;     // mag_key of the pivot
+struct __align__(16) Slot {
+    unsigned long long key;      // mag_key of the pivot
     int pos;                     // its place in the CTA's list of rows in use
     int row;                     // local row; bit 30: the pivot is exactly zero
-    T2 inv;                      // its reciprocal
+    double2 inv;                 // its reciprocal
 };
 
 constexpr int MAX_CLUSTER = 16;
 
-template <class T2> size_t smem_bytes(int n, int C) {
+inline size_t smem_bytes(int n, int C) {
     const int rl = (n + C - 1) / C;
-    return sizeof(T2) * ((size_t)rl * (n + 2) + n) + 16 + 2 * MAX_CLUSTER * sizeof(Slot<T2>) + sizeof(int) * 2 * rl;
+    return sizeof(double2) * ((size_t)rl * (n + 2) + n) + 16 + 2 * MAX_CLUSTER * sizeof(Slot) + sizeof(int) * 2 * rl;
 }
 
 __device__ __forceinline__ uint32_t cl_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
@@ -120,36 +113,34 @@ template <class T> __device__ __forceinline__ T* cl_map(T* p, uint32_t rank) {
 }
 
 // Where(e): {source, destination, row stride, perm, status} of energy e
-template <class T2> struct Place { const T2* S; T2* F; int ld; int* perm; int* status; };
+struct Place { const double2* S; double2* F; int ld; int* perm; int* status; };
 
 constexpr int ZERO_BIT = 1 << 30;
 
 // Warp 0: column c of the rows in use brought up to date (v -= l u over the multipliers lm of
 // the previous column; UPDATE false: as it stands), its best row found and proposed to every
 // CTA of the cluster.  Lanes 2q, 2q + 1: real and imaginary part of one row.
-template <class T2, bool UPDATE>
-__device__ __forceinline__ void propose(T2* rows, int ldr, int na, const int* ord, const T2* lm, T2 u, int C, uint32_t rank, int c,
-                                        Slot<T2>* slots, int par) {
-    using T = typename Real<T2>::t;
+template <bool UPDATE>
+__device__ __forceinline__ void propose(double2* rows, int ldr, int na, const int* ord, const double2* lm, double2 u, int C,
+                                        uint32_t rank, int c, Slot* slots, int par) {
     const int lane = threadIdx.x & 31, part = lane & 1;
-    using K = typename Key<T2>::t;
-    K bk = 0;
+    unsigned long long bk = 0;
     int bp = 0, br = 0;
-    T bx = T(1), by = T(0);
+    double bx = 1.0, by = 0.0;
     for (int q0 = 0; q0 < na; q0 += 16) {
         const int q = q0 + (lane >> 1);
         const bool in = q < na;
         const int r = ord[in ? q : 0];
-        T2* a = rows + (size_t)r * ldr + c;
-        T v = part ? a->y : a->x;
+        double2* a = rows + (size_t)r * ldr + c;
+        double v = part ? a->y : a->x;
         if (UPDATE) {
-            const T2 l = lm[r];
+            const double2 l = lm[r];
             // re: v - l.x u.x + l.y u.y;  im: v - l.x u.y - l.y u.x
             v = part ? fma(-l.x, u.y, fma(-l.y, u.x, v)) : fma(-l.x, u.x, fma(l.y, u.y, v));
-            if (in) reinterpret_cast<T*>(a)[part] = v;
+            if (in) reinterpret_cast<double*>(a)[part] = v;
         }
-        const T o = __shfl_xor_sync(0xffffffffu, v, 1);
-        const K k = in ? mag_key(fabs(v) + fabs(o)) : K(0);
+        const double o = __shfl_xor_sync(0xffffffffu, v, 1);
+        const unsigned long long k = in ? mag_key(fabs(v) + fabs(o)) : 0ull;
         if (q0 == 0 || k > bk) {
             bk = k;
             bp = q;
@@ -159,10 +150,10 @@ __device__ __forceinline__ void propose(T2* rows, int ldr, int na, const int* or
         }
     }
     // the reciprocals of the lanes' own candidates, beside the search
-    const bool zero = bx == T(0) && by == T(0);
-    const T2 inv = inverse(zero ? make2<T2>(T(1), T(0)) : make2<T2>(bx, by));
+    const bool zero = bx == 0.0 && by == 0.0;
+    const double2 inv = inverse(zero ? make_double2(1.0, 0.0) : make_double2(bx, by));
     const int win = warp_best(bk);
-    Slot<T2>* own = slots + par * MAX_CLUSTER + rank;
+    Slot* own = slots + par * MAX_CLUSTER + rank;
     if (lane == win) {
         own->key = bk;
         own->pos = bp;
@@ -171,25 +162,24 @@ __device__ __forceinline__ void propose(T2* rows, int ldr, int na, const int* or
     }
     if (C > 1) {
         __syncwarp();
-        const Slot<T2> s = *own;
+        const Slot s = *own;
         if (lane < C && lane != (int)rank) *cl_map(own, (uint32_t)lane) = s;
     }
 }
 
-template <class T2, class Where>
+template <class Where>
 __global__ void __launch_bounds__(256) k_lu(Where where, int n) {
-    using T = typename Real<T2>::t;
     extern __shared__ __align__(16) unsigned char lu_sm[];
     const uint32_t C = cl_size(), rank = cl_rank();
     const int e = blockIdx.x / C;
-    const Place<T2> P = where(e);
+    const Place P = where(e);
     const int rl_max = (n + (int)C - 1) / (int)C;
     const int rl = (n - (int)rank + (int)C - 1) / (int)C;      // rows of this CTA
     const int ldr = n + 1, NT = blockDim.x, t = threadIdx.x, warp = t >> 5, lane = t & 31, nw = NT >> 5;
-    T2* rows = reinterpret_cast<T2*>(lu_sm);
-    T2* urow = rows + (size_t)rl_max * ldr;                    // the pivot row
-    T2* lm = urow + n;                                         // multipliers of the local rows
-    Slot<T2>* slots = reinterpret_cast<Slot<T2>*>(lu_sm + (sizeof(T2) * ((size_t)rl_max * (ldr + 1) + n) + 15) / 16 * 16);
+    double2* rows = reinterpret_cast<double2*>(lu_sm);
+    double2* urow = rows + (size_t)rl_max * ldr;               // the pivot row
+    double2* lm = urow + n;                                    // multipliers of the local rows
+    Slot* slots = reinterpret_cast<Slot*>(lu_sm + (sizeof(double2) * ((size_t)rl_max * (ldr + 1) + n) + 15) / 16 * 16);
     int* step = reinterpret_cast<int*>(slots + 2 * MAX_CLUSTER);   // pivot step of a local row
     int* ord = step + rl_max;                                  // the rows not used yet: ord[0 .. na)
     for (int r = warp; r < rl; r += nw)
@@ -198,22 +188,21 @@ __global__ void __launch_bounds__(256) k_lu(Where where, int n) {
     int na = rl;
     __syncthreads();
     if (C > 1) cl_sync();       // every CTA runs before its shared memory is written from outside
-    if (warp == 0) propose<T2, false>(rows, ldr, na, ord, lm, make2<T2>(T(0), T(0)), (int)C, rank, 0, slots, 0);
+    if (warp == 0) propose<false>(rows, ldr, na, ord, lm, make_double2(0.0, 0.0), (int)C, rank, 0, slots, 0);
     int bad = 0;
     for (int j = 0; j < n; ++j) {
         if (C > 1) cl_sync();
         else __syncthreads();
         // the winner, by every warp on its own
-        const Slot<T2>* set = slots + (j & 1) * MAX_CLUSTER;
-        using K = typename Key<T2>::t;
-        const int w = C > 1 ? warp_best(lane < (int)C ? set[lane].key : K(0)) : 0;
+        const Slot* set = slots + (j & 1) * MAX_CLUSTER;
+        const int w = C > 1 ? warp_best(lane < (int)C ? set[lane].key : 0ull) : 0;
         const int lr = set[w].row & ~ZERO_BIT;
         bad |= set[w].row & ZERO_BIT;
-        const T2 inv = set[w].inv;
+        const double2 inv = set[w].inv;
         const bool mine = w == (int)rank;
         const int wpos = set[w].pos;
-        const T2* prow = (C > 1 ? cl_map(rows, (uint32_t)w) : rows) + (size_t)lr * ldr;
-        T2 pv[4];               // the pivot row on its way while the multipliers are made (n <= 1024)
+        const double2* prow = (C > 1 ? cl_map(rows, (uint32_t)w) : rows) + (size_t)lr * ldr;
+        double2 pv[4];          // the pivot row on its way while the multipliers are made (n <= 1024)
 #pragma unroll
         for (int x = 0; x < 4; ++x)
             if (j + 1 + t + x * NT < n) pv[x] = prow[j + 1 + t + x * NT];
@@ -221,11 +210,11 @@ __global__ void __launch_bounds__(256) k_lu(Where where, int n) {
         // lane reads and writes its own part only and has the other by shuffle
         for (int q0 = warp * 16; q0 < na; q0 += NT >> 1) {
             const int q = q0 + (lane >> 1), part = lane & 1, r = ord[min(q, na - 1)];
-            T* a = reinterpret_cast<T*>(rows + (size_t)r * ldr + j) + part;
-            const T v = q < na ? *a : T(0), o = __shfl_xor_sync(0xffffffffu, v, 1);
-            const T l = part ? fma(o, inv.y, v * inv.x) : fma(v, inv.x, -(o * inv.y));
+            double* a = reinterpret_cast<double*>(rows + (size_t)r * ldr + j) + part;
+            const double v = q < na ? *a : 0.0, o = __shfl_xor_sync(0xffffffffu, v, 1);
+            const double l = part ? fma(o, inv.y, v * inv.x) : fma(v, inv.x, -(o * inv.y));
             if (q < na && !(mine && r == lr)) {
-                reinterpret_cast<T*>(lm + r)[part] = l;
+                reinterpret_cast<double*>(lm + r)[part] = l;
                 *a = l;
             }
         }
@@ -242,42 +231,21 @@ __global__ void __launch_bounds__(256) k_lu(Where where, int n) {
             __syncthreads();
         }
         if (j + 1 == n) break;
-        if (warp == 0) propose<T2, true>(rows, ldr, na, ord, lm, urow[j + 1], (int)C, rank, j + 1, slots, (j + 1) & 1);
+        if (warp == 0) propose<true>(rows, ldr, na, ord, lm, urow[j + 1], (int)C, rank, j + 1, slots, (j + 1) & 1);
         // A[r][c] -= l[r] u[c] over the rows in use and columns past j + 1; warp 0 joins when
         // it has proposed
         const int cols = n - j - 2;
-        if (sizeof(T) == 8) {
-            // items across row ends, so that no lane of a 64-cycle instruction is idle
-            for (int q = (warp + nw - 1) % nw * 32 + lane; q < cols * na; q += NT) {
-                const int r = ord[q / cols], c = j + 2 + q % cols;
-                T2* a = rows + (size_t)r * ldr + c;
-                *a = fnma(*a, lm[r], urow[c]);
-            }
-        } else {
-            constexpr int RG = 8;       // rows at a time, loads before stores
-            const int segs = (cols + 31) / 32, groups = (na + RG - 1) / RG;
-            for (int q = (warp + nw - 1) % nw; q < segs * groups; q += nw) {
-                const int c = min(j + 2 + q / groups * 32 + lane, n - 1), g = q % groups * RG;
-                const bool in = j + 2 + q / groups * 32 + lane < n;
-                const T2 u = urow[c];
-                T2* a[RG];
-                T2 v[RG];
-#pragma unroll
-                for (int x = 0; x < RG; ++x) {
-                    const int r = ord[min(g + x, na - 1)];
-                    a[x] = rows + (size_t)r * ldr + c;
-                    v[x] = fnma(*a[x], lm[r], u);
-                }
-#pragma unroll
-                for (int x = 0; x < RG; ++x)
-                    if (in && g + x < na) *a[x] = v[x];
-            }
+        // items across row ends, so that no lane of a 64-cycle instruction is idle
+        for (int q = (warp + nw - 1) % nw * 32 + lane; q < cols * na; q += NT) {
+            const int r = ord[q / cols], c = j + 2 + q % cols;
+            double2* a = rows + (size_t)r * ldr + c;
+            *a = fnma(*a, lm[r], urow[c]);
         }
     }
     if (C > 1) cl_sync();       // no CTA leaves while its rows may be read; all reads of S are done
     for (int r = warp; r < rl; r += nw) {
         const int j = step[r];
-        T2* out = P.F + (size_t)j * P.ld;
+        double2* out = P.F + (size_t)j * P.ld;
         for (int c = lane; c < n; c += 32) out[c] = rows[(size_t)r * ldr + c];
         if (lane == 0) P.perm[j] = r * (int)C + (int)rank;
     }
@@ -286,18 +254,15 @@ __global__ void __launch_bounds__(256) k_lu(Where where, int n) {
 
 // Cluster size for nb blocks of n x n: the one with the least waves x max(chain, update).
 // 0: no size holds the rows in shared memory.  Chain and update per column in cycles, from
-// the measurements above: FP64 1300 on one CTA, 1700 across a cluster, 2 per element of
-// update; FP32 450, 900 and 0.16.
-template <class T2, class Where> int pick_cluster(int n, int nb, int sms, int smem_max) {
-    const bool f64 = sizeof(T2) == 16;
-    const double alpha = f64 ? 2.0 : 0.16;
+// the measurements above: 1300 on one CTA, 1700 across a cluster, 2 per element of update.
+template <class Where> int pick_cluster(int n, int nb, int sms, int smem_max) {
     int best = 0;
     double tb = 0;
     for (int C = 1; C <= MAX_CLUSTER; C *= 2) {
-        const size_t sm = smem_bytes<T2>(n, C);
+        const size_t sm = smem_bytes(n, C);
         if (sm > (size_t)smem_max || C > n) continue;
-        cudaFuncSetAttribute(k_lu<T2, Where>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-        cudaFuncSetAttribute(k_lu<T2, Where>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute(k_lu<Where>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+        cudaFuncSetAttribute(k_lu<Where>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaLaunchConfig_t cf{};
         cudaLaunchAttribute at{};
         cf.gridDim = dim3(C);
@@ -309,28 +274,28 @@ template <class T2, class Where> int pick_cluster(int n, int nb, int sms, int sm
         cf.attrs = &at;
         cf.numAttrs = 1;
         int fit = 0;
-        if (cudaOccupancyMaxActiveClusters(&fit, k_lu<T2, Where>, &cf) != cudaSuccess || fit < 1) { cudaGetLastError(); continue; }
+        if (cudaOccupancyMaxActiveClusters(&fit, k_lu<Where>, &cf) != cudaSuccess || fit < 1) { cudaGetLastError(); continue; }
         const int run = std::min(nb, fit), waves = (nb + fit - 1) / fit, share = (run * C + sms - 1) / sms;
-        const double chain = C == 1 ? (f64 ? 1300 : 450) : (f64 ? 1700 : 900);
-        const double tt = waves * std::max(chain, (double)n * n / (3.0 * C) * alpha * share);
+        const double chain = C == 1 ? 1300 : 1700;
+        const double tt = waves * std::max(chain, (double)n * n / (3.0 * C) * 2.0 * share);
         if (!best || tt < tb) { best = C; tb = tt; }
     }
     return best;
 }
 
-template <class T2, class Where> cudaError_t launch(const Where& where, int n, int nb, int C, cudaStream_t st) {
+template <class Where> cudaError_t launch(const Where& where, int n, int nb, int C, cudaStream_t st) {
     cudaLaunchConfig_t cf{};
     cudaLaunchAttribute at{};
     cf.gridDim = dim3(C * nb);
     cf.blockDim = dim3(256);
-    cf.dynamicSmemBytes = smem_bytes<T2>(n, C);
+    cf.dynamicSmemBytes = smem_bytes(n, C);
     cf.stream = st;
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = C;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cf.attrs = &at;
     cf.numAttrs = 1;
-    return cudaLaunchKernelEx(&cf, k_lu<T2, Where>, where, n);
+    return cudaLaunchKernelEx(&cf, k_lu<Where>, where, n);
 }
 
 }  // namespace lu

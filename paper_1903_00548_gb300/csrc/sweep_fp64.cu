@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(256) k_node(SweepSys sys, const SweepJob* __re
 struct Where64 {
     const SweepJob* jobs;
     SweepSys sys;
-    __device__ lu::Place<double2> operator()(int e) const {
+    __device__ lu::Place operator()(int e) const {
         const SweepJob& J = jobs[e];
         return {J.S, J.S, sys.n, perm_of(sys, J), J.status};
     }
@@ -897,7 +897,7 @@ int sweep_tiled(const SweepSys& sys, const SweepJob* jobs, const SweepJob* host,
         const int yc = GREEN ? 0 : (last ? m : ms);
         if (big) k_node<2, GREEN><<<dim3(t32 + (yc + 31) / 32, t32, nb), 256, 0, st>>>(sys, jobs, i);
         else k_node<1, GREEN><<<dim3(t16 + (yc + 15) / 16, t16, nb), 256, 0, st>>>(sys, jobs, i);
-        lu::launch<double2>(where, n, nb, C, st);
+        lu::launch(where, n, nb, C, st);
         launches += 2;
         const int cols = (last ? 0 : n) + (GREEN ? n : yc);
         if (cols > 0) {
@@ -937,7 +937,7 @@ int sweep_any(const SweepSys& sys, const SweepJob* jobs, const SweepJob* host, i
         k_sweep_small<<<nb, 128, small_smem(sys.n, m), st>>>(sys, jobs);
         return 1;
     }
-    const int C = lu::pick_cluster<double2, Where64>(sys.n, nb, sms, smem_max);
+    const int C = lu::pick_cluster<Where64>(sys.n, nb, sms, smem_max);
     // the solve's shared memory for 4 columns is below the factorisation's limit at any n that has a cluster
     if (C > 0 && nb <= 65535 && solve_smem(sys.n, 4) <= (size_t)smem_max) return sweep_tiled<GREEN>(sys, jobs, host, nb, C, sms, smem_max, st);
     k_sweep_fp64<GREEN><<<nb, NT, 0, st>>>(sys, jobs);
