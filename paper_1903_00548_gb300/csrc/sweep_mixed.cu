@@ -984,61 +984,61 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
         const C64Sweep cs{sys, jobs_d, m, w, S.F, S.sF, S.piv, S.sP, S.XY, S.sXY, S.Lb, S.sL, S.C64, S.sC};
         c->launches += c64_sweep(cs, jobs.data(), nb, c->sm_count, smem_optin, st);
     } else {
-    const int fblocks = (int)std::min<size_t>(((size_t)n * n + NT - 1) / NT, 512);
-    const size_t panel_smem = sizeof(float2) * (size_t)(n + 1) * PW;
-    if (panel_smem > (size_t)smem_optin)
-        return fail(c, PWQT_ERR_INVALID_ARG, "the complex64 panel of block size " + std::to_string(n) +
-                                                 " exceeds shared memory: use PWQT_FP64 (mixed precision takes n <= " +
-                                                 std::to_string(smem_optin / (int)(sizeof(float2) * PW) - 1) + ")");
-    // the limit is a property of the kernel, shared by every context in the process (several
-    // contexts on several host threads run here at once): always the device maximum, never a
-    // per-call value that another thread could lower under a launch in flight
-    cudaFuncAttributes fa_panel{};
-    PWQT_CUDA(c, cudaFuncGetAttributes(&fa_panel, k_mx_panel));
-    // the opt-in maximum counts static and dynamic shared memory together
-    const int dyn_panel = smem_optin - (int)fa_panel.sharedSizeBytes;
-    if (panel_smem > (size_t)dyn_panel) return fail(c, PWQT_ERR_INVALID_ARG, "panel exceeds shared memory");
-    PWQT_CUDA(c, cudaFuncSetAttribute(k_mx_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_panel));
-    auto gemm = [&](const float2* A, long long sA, int lda, const float2* B1, long long sB1, int ldb1, const float2* B2, long long sB2,
-                    int ldb2, float2* C1, long long sC1, int ldc1, float2* C2, long long sC2, int ldc2, int split, int M, int Nc, int K) {
-        CGemmArgs g{A, sA, lda, B1, sB1, ldb1, B2, sB2, ldb2, C1, sC1, ldc1, C2, sC2, ldc2, split};
-        launch_cgemm_tc(g, nb, M, Nc, K, st);
-        c->launches++;
-    };
-    for (int i = 0; i < N; ++i) {
-        float2* Fi = S.F + (size_t)i * n * n;
-        float2* XYi = S.XY + (size_t)i * n * w;
-        k_mx_form<<<dim3(fblocks, nb), NT, 0, st>>>(S, i);
-        c->launches++;
-        if (i > 0) {
-            const float2* XYp = S.XY + (size_t)(i - 1) * n * w;
-            gemm(S.Lb + (size_t)i * n * n, S.sL, n, XYp, S.sXY, w, XYp + n, S.sXY, w, Fi, S.sF, n, XYi + n, S.sXY, w, n, n, w, n);
-        }
-        for (int k0 = 0; k0 < n; k0 += PW) {
-            const int wd = std::min(PW, n - k0);
-            if (n - k0 <= 2 * PR_NT) k_mx_panel_reg<<<nb, PR_NT, 0, st>>>(S, i, k0, wd);
-            else k_mx_panel<<<nb, NT, sizeof(float2) * (size_t)((n - k0) | 1) * PW, st>>>(S, i, k0, wd);
-            k_mx_panel_apply<<<dim3((n - wd + w + APT - 1) / APT, nb), APT, 0, st>>>(S, i, k0, wd);
-            c->launches += 2;
-            const int rest = n - k0 - wd;
-            if (rest > 0)
-                gemm(Fi + (size_t)(k0 + wd) * n + k0, S.sF, n, Fi + (size_t)k0 * n + k0 + wd, S.sF, n, XYi + (size_t)k0 * w, S.sXY, w,
-                     Fi + (size_t)(k0 + wd) * n + k0 + wd, S.sF, n, XYi + (size_t)(k0 + wd) * w, S.sXY, w, rest, rest, rest + w, wd);
-        }
-        for (int k0 = ((n - 1) / PW) * PW; k0 >= 0; k0 -= PW) {
-            const int wd = std::min(PW, n - k0);
-            k_mx_trsm_up<<<dim3((w + APT - 1) / APT, nb), APT, 0, st>>>(S, i, k0, wd);
+        const int fblocks = (int)std::min<size_t>(((size_t)n * n + NT - 1) / NT, 512);
+        const size_t panel_smem = sizeof(float2) * (size_t)(n + 1) * PW;
+        if (panel_smem > (size_t)smem_optin)
+            return fail(c, PWQT_ERR_INVALID_ARG, "the complex64 panel of block size " + std::to_string(n) +
+                                                     " exceeds shared memory: use PWQT_FP64 (mixed precision takes n <= " +
+                                                     std::to_string(smem_optin / (int)(sizeof(float2) * PW) - 1) + ")");
+        // the limit is a property of the kernel, shared by every context in the process (several
+        // contexts on several host threads run here at once): always the device maximum, never a
+        // per-call value that another thread could lower under a launch in flight
+        cudaFuncAttributes fa_panel{};
+        PWQT_CUDA(c, cudaFuncGetAttributes(&fa_panel, k_mx_panel));
+        // the opt-in maximum counts static and dynamic shared memory together
+        const int dyn_panel = smem_optin - (int)fa_panel.sharedSizeBytes;
+        if (panel_smem > (size_t)dyn_panel) return fail(c, PWQT_ERR_INVALID_ARG, "panel exceeds shared memory");
+        PWQT_CUDA(c, cudaFuncSetAttribute(k_mx_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_panel));
+        auto gemm = [&](const float2* A, long long sA, int lda, const float2* B1, long long sB1, int ldb1, const float2* B2, long long sB2,
+                        int ldb2, float2* C1, long long sC1, int ldc1, float2* C2, long long sC2, int ldc2, int split, int M, int Nc, int K) {
+            CGemmArgs g{A, sA, lda, B1, sB1, ldb1, B2, sB2, ldb2, C1, sC1, ldc1, C2, sC2, ldc2, split};
+            launch_cgemm_tc(g, nb, M, Nc, K, st);
             c->launches++;
-            if (k0 > 0) gemm(Fi + k0, S.sF, n, XYi + (size_t)k0 * w, S.sXY, w, XYi + (size_t)k0 * w, S.sXY, w, XYi, S.sXY, w, XYi, S.sXY,
-                             w, w, k0, w, wd);
+        };
+        for (int i = 0; i < N; ++i) {
+            float2* Fi = S.F + (size_t)i * n * n;
+            float2* XYi = S.XY + (size_t)i * n * w;
+            k_mx_form<<<dim3(fblocks, nb), NT, 0, st>>>(S, i);
+            c->launches++;
+            if (i > 0) {
+                const float2* XYp = S.XY + (size_t)(i - 1) * n * w;
+                gemm(S.Lb + (size_t)i * n * n, S.sL, n, XYp, S.sXY, w, XYp + n, S.sXY, w, Fi, S.sF, n, XYi + n, S.sXY, w, n, n, w, n);
+            }
+            for (int k0 = 0; k0 < n; k0 += PW) {
+                const int wd = std::min(PW, n - k0);
+                if (n - k0 <= 2 * PR_NT) k_mx_panel_reg<<<nb, PR_NT, 0, st>>>(S, i, k0, wd);
+                else k_mx_panel<<<nb, NT, sizeof(float2) * (size_t)((n - k0) | 1) * PW, st>>>(S, i, k0, wd);
+                k_mx_panel_apply<<<dim3((n - wd + w + APT - 1) / APT, nb), APT, 0, st>>>(S, i, k0, wd);
+                c->launches += 2;
+                const int rest = n - k0 - wd;
+                if (rest > 0)
+                    gemm(Fi + (size_t)(k0 + wd) * n + k0, S.sF, n, Fi + (size_t)k0 * n + k0 + wd, S.sF, n, XYi + (size_t)k0 * w, S.sXY, w,
+                         Fi + (size_t)(k0 + wd) * n + k0 + wd, S.sF, n, XYi + (size_t)(k0 + wd) * w, S.sXY, w, rest, rest, rest + w, wd);
+            }
+            for (int k0 = ((n - 1) / PW) * PW; k0 >= 0; k0 -= PW) {
+                const int wd = std::min(PW, n - k0);
+                k_mx_trsm_up<<<dim3((w + APT - 1) / APT, nb), APT, 0, st>>>(S, i, k0, wd);
+                c->launches++;
+                if (k0 > 0) gemm(Fi + k0, S.sF, n, XYi + (size_t)k0 * w, S.sXY, w, XYi + (size_t)k0 * w, S.sXY, w, XYi, S.sXY, w, XYi, S.sXY,
+                                 w, w, k0, w, wd);
+            }
         }
-    }
-    // node back substitution c_i = y_i - X_i c_{i+1}
-    for (int i = N - 2; i >= 0; --i) {
-        float2* XYi = S.XY + (size_t)i * n * w;
-        const float2* XYn = S.XY + (size_t)(i + 1) * n * w;
-        gemm(XYi, S.sXY, w, XYn + n, S.sXY, w, XYn + n, S.sXY, w, XYi + n, S.sXY, w, XYi + n, S.sXY, w, m, n, m, n);
-    }
+        // node back substitution c_i = y_i - X_i c_{i+1}
+        for (int i = N - 2; i >= 0; --i) {
+            float2* XYi = S.XY + (size_t)i * n * w;
+            const float2* XYn = S.XY + (size_t)(i + 1) * n * w;
+            gemm(XYi, S.sXY, w, XYn + n, S.sXY, w, XYn + n, S.sXY, w, XYi + n, S.sXY, w, XYi + n, S.sXY, w, m, n, m, n);
+        }
     }
     if (c->profile) {
         PWQT_CUDA(c, cudaEventRecord(L.ev[1], st));
