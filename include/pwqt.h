@@ -56,8 +56,9 @@ typedef struct pwqt_ctx pwqt_ctx;
 
 /* precision of the block sweep */
 #define PWQT_FP64                0    /* complex128 throughout                     */
-#define PWQT_MIXED               1    /* complex64 factorisation on the tensor
-                                         cores (3xTF32 products, FP32 accumulate)
+#define PWQT_MIXED               1    /* complex64 factorisation (block sizes 25 to
+                                         320 on the FP32 pipes, others on the tensor
+                                         cores with 3xTF32 products, FP32 accumulate)
                                          + refinement with FP64-accurate residuals
                                          (see pwqt_set_residual)                   */
 #define PWQT_FP32                2    /* the complex64 factorisation alone (no

@@ -4,9 +4,9 @@
 // The columns are dealt out in blocks of 8 (block b to CTA b % C) and stay in shared
 // memory, row r of a block in 64 consecutive bytes; a factored panel takes its block's place
 // column by column (a lane per row stores without bank conflicts, which rows of 64 bytes
-// would cost 400 cycles a column).  The owner of the next panel brings it
-// up to date, then one warp factors it in registers (RPL rows a lane, 8 columns each) while
-// the other warps update the remaining blocks with the panel before.  Rows are not moved: a
+// would cost 400 cycles a column).  The owner of the next panel brings it up to date, then
+// up to 4 warps factor it in registers (RPL rows a lane, 8 columns each) while the other
+// warps update the remaining blocks with the panel before.  Rows are not moved: a
 // row that has served as pivot is left alone and its part of U goes to the output as soon
 // as it is known; at the end row r of L is written where its pivot step says.  Factors of
 // P A with partial pivoting (max |re| + |im|), unit lower triangle, (P x)_j = x[perm[j]].
