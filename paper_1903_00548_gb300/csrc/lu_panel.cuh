@@ -286,7 +286,12 @@ __global__ void __launch_bounds__(NT) k_lu_panel(Batch B, int n) {
 // CTAs per energy; 0: none holds the block.  One CTA's updates keep up with the panel chain
 // to n = 80; above, they are spread over 4 (measured, 16 energies: n = 128 121 us on one CTA,
 // 104 on 2, 92 on 4, 107 on 8; n = 256 293 us on 4, 343 on 8: a larger cluster pays for the
-// panel's copy and the cluster barrier).
+// panel's copy and the cluster barrier; a whole mixed solve of 30 nodes on 4 against 8: 32
+// energies n = 256 74.3 and 75.5 ms, n = 320 121 and 138, but one energy 17.0 and 16.7, 26.0
+// and 25.5).
+// 320 is where the form's tests end, not where it stops paying: with 3 rows a lane and 8 CTAs
+// (shared memory holds n <= 440 or so) a mixed solve of 30 nodes takes, against the tensor-core
+// form, 16 energies n = 340 96 and 118 ms, n = 384 119 and 151; one energy 29 and 61, 38 and 74.
 inline int pick_cluster(int n, int smem_max) {
     if (n > 320) return 0;
     for (int C = n <= 80 ? 1 : 4; C <= 8; C *= 2)

@@ -17,7 +17,8 @@ namespace pwqt {
 // node density n[i][c] = sum_{gamma in c} (2/|v_gamma|) sum_alpha |c_{i alpha gamma}|^2.
 // ntd ms + nts m inner products of length n per energy, FP64-bound: dealt out to OBS_CTAS
 // CTAs per energy, a warp per out-mode with its lanes along the injected modes (one
-// energy's CTA took 0.6 ms at n = 128 and 77 modes when it did them alone).  The CTAs'
+// energy's CTA took 0.6 ms at n = 128 and 77 modes when it did them alone); 38 so that four
+// energies fill the 152 SMs, more energies queue (8 of them 0.11 ms at n = 128).  The CTAs'
 // sums meet in the outputs, which the caller has zeroed.
 constexpr int OBS_CTAS = 38;
 __global__ void __launch_bounds__(256) k_observables(int n, int N, const ObsJob* __restrict__ jobs) {

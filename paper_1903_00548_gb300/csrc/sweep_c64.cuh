@@ -19,7 +19,9 @@ struct C64Sweep {
 };
 
 // whether the block size has this form on a device with smem_max bytes of shared memory a CTA
-// (25 .. 320: below, one tensor-core tile takes a whole node product and a panel the block)
+// (25 .. 320, the sizes that its tests cover.  It is the faster one beyond both ends too: mixed
+// solve of 60 nodes and 32 energies, tensor-core form and this, n = 8 6.2 and 2.4 ms, n = 16 7.4
+// and 3.3, n = 24 8.7 and 4.2; above 320 see lup::pick_cluster)
 bool c64_sweep_fits(int n, int smem_max);
 // factors, couplings, X_i and the solution of nb energies (jobs; host: the same table on the
 // host); returns the number of kernels launched

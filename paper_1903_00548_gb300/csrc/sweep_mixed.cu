@@ -977,7 +977,7 @@ int solve_mixed(pwqt_ctx* c, System& s, const SweepSys& sys, std::vector<SweepJo
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->dev);
     // up to block 320 a small cluster's shared memory holds the node block and the FP32 pipes
     // beat the tensor-core form: three launches a node against 5 n / 32 (sweep of 16 energies
-    // at n = 128, 50 nodes: 57 -> 13 ms)
+    // at n = 128, 50 nodes: 57 -> 14 ms)
     const bool small = c64_sweep_fits(n, smem_optin);
     if (c->profile) PWQT_CUDA(c, cudaEventRecord(L.ev[0], st));
     if (small) {
