@@ -206,16 +206,18 @@ __global__ void __launch_bounds__(256) k_lu(Where where, int n) {
 #pragma unroll
         for (int x = 0; x < 4; ++x)
             if (j + 1 + t + x * NT < n) pv[x] = prow[j + 1 + t + x * NT];
-        // multipliers l = a inv, lanes 2q and 2q + 1 the real and imaginary part of one row's: a
-        // lane reads and writes its own part only and has the other by shuffle
+        // multipliers l = a inv, lanes 2q and 2q + 1 the real and imaginary part of one row's: both
+        // read the entry, and the warp, whole in every pass, is past its reads before either
+        // part is written (an exchange of the parts by shuffle instead: 0.7 % of a call at n = 64)
         for (int q0 = warp * 16; q0 < na; q0 += NT >> 1) {
             const int q = q0 + (lane >> 1), part = lane & 1, r = ord[min(q, na - 1)];
-            double* a = reinterpret_cast<double*>(rows + (size_t)r * ldr + j) + part;
-            const double v = q < na ? *a : 0.0, o = __shfl_xor_sync(0xffffffffu, v, 1);
-            const double l = part ? fma(o, inv.y, v * inv.x) : fma(v, inv.x, -(o * inv.y));
+            double2* a = rows + (size_t)r * ldr + j;
+            const double2 v = *a;
+            const double l = part ? fma(v.x, inv.y, v.y * inv.x) : fma(v.x, inv.x, -(v.y * inv.y));
+            __syncwarp();
             if (q < na && !(mine && r == lr)) {
                 reinterpret_cast<double*>(lm + r)[part] = l;
-                *a = l;
+                reinterpret_cast<double*>(a)[part] = l;
             }
         }
 #pragma unroll
